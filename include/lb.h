@@ -140,7 +140,10 @@ lb_status lb_trace(lb_state* s, double* buf, int cap, int* count);
  *      multiple of 32 and nx >= block_x + 64).
  * lb_init starts with pipeline 0 (measured the faster of the two on GB300 for
  * the 8192 x 8192 lattice). rows_per_cta is in
- * [4, 4096]. The shape changes how the work is split, not the trajectory;
+ * [4, 4096]. With pipeline 0 the shape is that of the steps taken one at a time
+ * (those that append a trace row, and a last odd one); lb_step takes other steps
+ * two at a time through a kernel with a shape of its own.
+ * The shape changes how the work is split, not the trajectory;
  * only the FP32 rounding of the energy partial sums depends on it.
  * Errors: LB_ERR_ARG for NULL or unsupported values, LB_ERR_STATE for an FP64
  * state (whose kernels have no such shape). */

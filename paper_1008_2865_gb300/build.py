@@ -23,6 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 UNITS = {
     "lb_api.cu": [],
     "lb_fp32.cu": [],
+    "lb_pair.cu": [],
     "lb_bulk.cu": [],
     "lb_batch.cu": [],
     "lb_adjoint.cu": [],

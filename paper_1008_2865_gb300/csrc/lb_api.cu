@@ -236,6 +236,19 @@ lb_status step_fp32(lb_state* s, long n)
         const bool reduce = s->p.trace_every > 0 && (s->t % s->p.trace_every) == 0;
         cudaError_t e;
         const bool bulk = s->launch.pipeline == 1;
+        // two steps without a trace row of their own go through the lattice together
+        // (lb_pair.cu): the same fields bit for bit, half the memory traffic
+        const bool next_reduces =
+            s->p.trace_every > 0 && ((s->t + 1) % s->p.trace_every) == 0;
+        if (!bulk && !reduce && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
+            e = s->p.prec == LB_FP32 ? fp32_step_pair(make_args<float>(s), s->stream)
+                                     : fp16_step_pair(make_args<__half>(s), s->stream);
+            if (e != cudaSuccess) return fail_cuda(s);
+            s->cur ^= 1;
+            s->t += 2;
+            ++k;
+            continue;
+        }
         if (s->p.prec == LB_FP32)
             e = bulk ? fp32_step_bulk(make_args<float>(s), s->launch, reduce, s->stream)
                      : fp32_step(make_args<float>(s), s->launch, reduce, s->stream);

@@ -161,6 +161,12 @@ struct BatchLaunch {
 };
 cudaError_t fp32_batch_step(const BatchLaunch<float>& b, bool reduce, cudaStream_t s);
 cudaError_t fp16_batch_step(const BatchLaunch<__half>& b, bool reduce, cudaStream_t s);
+// Two plain steps in one pass (lb_pair.cu), for lattices of 2^18 sites on: below, its
+// few long chunks take as long as two launches of k_step (us per step, single and
+// paired: 250x187 10.1 and 10.2, 512^2 10.3 and 9.3, 700^2 12.3 and 10.2).
+inline bool pairs_pay(long long n) { return n >= (1LL << 18); }
+cudaError_t fp32_step_pair(const StepArgs<float>& a, cudaStream_t s);
+cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s);
 // bulk-copy pipelined step (lb_bulk.cu)
 bool bulk_supported(int nx, int ny, int elem_bytes, int block_x);
 int bulk_grid_blocks(int nx, int ny, int elem_bytes, Fp32Launch L);
