@@ -431,7 +431,9 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
     if (C < 1) C = 1;
     const long long K = T > 0 ? (T + C - 1) / C : 0;     // checkpoints at t = 0, C, 2C, ...
     const size_t GE = (size_t)g_elems(s->p.nx, s->p.ny);
-    const size_t slot = GE + (size_t)N;                   // populations (GE) then dpsi (N), floats
+    // populations (GE floats) then dpsi (N), rounded up so that every state starts
+    // 256-byte aligned: the populations are read in pairs, and N may be odd
+    const size_t slot = (GE + (size_t)N + 63) / 64 * 64;
     cudaStream_t st = s->stream;
 
     // ---- working memory of one call (freed on return): checkpoints, two segment
