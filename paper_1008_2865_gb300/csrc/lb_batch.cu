@@ -34,10 +34,14 @@ struct lb_batch {
     int nrows = 0;
     double* d_partials = nullptr;
     BatchRep* d_reps = nullptr;
-    // graph of one period of steps, starting at t % period == 0
+    int4* d_pair_tiles = nullptr;   // work list of the steps taken two at a time (lb_pair.cu)
+    int npair_tiles = 0;
+    bool odd = false;               // some replica has an odd nx
+    // graphs of one period of steps, starting at t % period == 0 with buffers 0 or 1 in
     cudaStream_t cap = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};
     int period = 0;
+    int period_flips = 0;           // 1 if a period ends with the buffers swapped
 };
 
 namespace {
@@ -45,7 +49,7 @@ namespace {
 void free_tables(lb_batch* b)
 {
     void* ptrs[] = {b->d_args[0], b->d_args[1], b->d_tiles, b->d_partials, b->d_reps,
-                    b->d_rowmap};
+                    b->d_rowmap, b->d_pair_tiles};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     b->d_args[0] = b->d_args[1] = nullptr;
@@ -53,8 +57,11 @@ void free_tables(lb_batch* b)
     b->d_rowmap = nullptr;
     b->d_partials = nullptr;
     b->d_reps = nullptr;
-    if (b->exec) cudaGraphExecDestroy(b->exec);
-    b->exec = nullptr;
+    b->d_pair_tiles = nullptr;
+    for (cudaGraphExec_t& e : b->exec) {
+        if (e) cudaGraphExecDestroy(e);
+        e = nullptr;
+    }
     cudaGetLastError();
 }
 
@@ -107,6 +114,11 @@ lb_status build_tables(lb_batch* b)
     }
     b->ntiles = (int)tiles.size();
     b->nrows = nrows_total;
+    std::vector<std::pair<int, int>> sizes;
+    for (const lb_state* s : b->reps) sizes.emplace_back(s->p.nx, s->p.ny);
+    std::vector<int4> pair_list;
+    pair_tiles(sizes, (int)elem_size(b->prec), b->om1, b->num_sms, pair_list);
+    b->npair_tiles = (int)pair_list.size();
     for (BatchRep& ri : info) ri.first_row += b->ntiles;
     const bool ok =
         (b->prec == LB_FP32 ? upload_args<float>(b) : upload_args<__half>(b)) &&
@@ -117,6 +129,9 @@ lb_status build_tables(lb_batch* b)
             cudaSuccess &&
         cudaMalloc((void**)&b->d_rowmap, sizeof(int2) * rowmap.size()) == cudaSuccess &&
         cudaMemcpy(b->d_rowmap, rowmap.data(), sizeof(int2) * rowmap.size(),
+                   cudaMemcpyHostToDevice) == cudaSuccess &&
+        cudaMalloc((void**)&b->d_pair_tiles, sizeof(int4) * pair_list.size()) == cudaSuccess &&
+        cudaMemcpy(b->d_pair_tiles, pair_list.data(), sizeof(int4) * pair_list.size(),
                    cudaMemcpyHostToDevice) == cudaSuccess &&
         cudaMalloc((void**)&b->d_reps, sizeof(BatchRep) * info.size()) == cudaSuccess &&
         cudaMemcpy(b->d_reps, info.data(), sizeof(BatchRep) * info.size(),
@@ -129,35 +144,50 @@ lb_status build_tables(lb_batch* b)
     return LB_OK;
 }
 
-// Enqueue step t (buffers `cur` in) of every replica on stream s.
-cudaError_t enqueue_step(const lb_batch* b, cudaStream_t s, long long t, int cur)
+template <typename T>
+BatchLaunch<T> batch_launch(const lb_batch* b, int cur)
 {
-    const bool reduce = b->trace_every > 0 && t % b->trace_every == 0;
-    if (b->prec == LB_FP32) {
-        BatchLaunch<float> L{static_cast<const StepArgs<float>*>(b->d_args[cur]), b->d_tiles,
-                             b->ntiles, b->d_partials, b->d_reps, (int)b->reps.size(),
-                             b->d_rowmap, b->nrows, b->block_x, b->om1, b->trace_every,
-                             b->num_sms, b->alternate};
-        return fp32_batch_step(L, reduce, s);
-    }
-    BatchLaunch<__half> L{static_cast<const StepArgs<__half>*>(b->d_args[cur]), b->d_tiles,
+    return BatchLaunch<T>{static_cast<const StepArgs<T>*>(b->d_args[cur]), b->d_tiles,
                           b->ntiles, b->d_partials, b->d_reps, (int)b->reps.size(),
                           b->d_rowmap, b->nrows, b->block_x, b->om1, b->trace_every,
                           b->num_sms, b->alternate};
-    return fp16_batch_step(L, reduce, s);
 }
 
-// Capture one period of steps starting at an aligned time (t % period == 0,
-// hence buffers 0 in) into a graph.
-bool build_graph(lb_batch* b)
+// Enqueue step t (buffers `cur` in) of every replica on stream s, or steps t and t + 1
+// together when `left` allows and neither appends a trace row; returns through `taken`
+// how many steps that was. Either way the buffers swap once.
+cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cur, long long left,
+                          int& taken)
 {
-    if (b->exec) return true;
+    const int te = b->trace_every;
+    const bool reduce = te > 0 && t % te == 0;
+    const bool next_reduces = te > 0 && (t + 1) % te == 0;
+    taken = !reduce && !next_reduces && left >= 2 ? 2 : 1;
+    if (b->prec == LB_FP32) {
+        const BatchLaunch<float> L = batch_launch<float>(b, cur);
+        return taken == 2 ? fp32_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, s)
+                          : fp32_batch_step(L, reduce, s);
+    }
+    const BatchLaunch<__half> L = batch_launch<__half>(b, cur);
+    return taken == 2 ? fp16_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, s)
+                      : fp16_batch_step(L, reduce, s);
+}
+
+// Capture one period of steps starting at an aligned time (t % period == 0) with
+// buffers `cur` in into a graph.
+bool build_graph(lb_batch* b, int cur)
+{
+    if (b->exec[cur]) return true;
     if (cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < b->period && e == cudaSuccess; ++k) e = enqueue_step(b, b->cap, k, k & 1);
+    int in = cur;
+    for (int k = 0, taken = 0; k < b->period && e == cudaSuccess; k += taken) {
+        e = enqueue_steps(b, b->cap, k, in, b->period - k, taken);
+        in ^= 1;
+    }
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e != cudaSuccess || e2 != cudaSuccess || !g) {
@@ -165,13 +195,14 @@ bool build_graph(lb_batch* b)
         cudaGetLastError();
         return false;
     }
-    const cudaError_t e3 = cudaGraphInstantiate(&b->exec, g, 0);
+    const cudaError_t e3 = cudaGraphInstantiate(&b->exec[cur], g, 0);
     cudaGraphDestroy(g);
     if (e3 != cudaSuccess) {
-        b->exec = nullptr;
+        b->exec[cur] = nullptr;
         cudaGetLastError();
         return false;
     }
+    b->period_flips = cur ^ in;
     return true;
 }
 
@@ -218,6 +249,7 @@ lb_status lb_batch_init(lb_batch** out, int count, const lb_params* params,
         b->reps.push_back(s);
         b->om1 = b->om1 && params[r].omega == 1.0;
         b->alternate = b->alternate || marches_alternate(s->N);
+        b->odd = b->odd || (s->p.nx & 1);
     }
     DeviceScope dev(b->device);
     if (!dev.ok ||
@@ -229,7 +261,7 @@ lb_status lb_batch_init(lb_batch** out, int count, const lb_params* params,
         return LB_ERR_CUDA;
     }
     const int te = b->trace_every;
-    b->period = te == 0 ? 2 : (te % 2 == 0 ? te : 2 * te);
+    b->period = te == 0 ? 16 : te < 8 ? (7 + te) / te * te : te;   // at least 8 steps
     if (b->period > 1024) b->period = 0;   // long periods: direct launches only
     const lb_status st = build_tables(b);
     if (st != LB_OK) {
@@ -249,15 +281,18 @@ lb_status lb_batch_step(lb_batch* b, long n)
     if (!dev.ok) return poison(b);
     while (n > 0) {
         if (b->use_graph && b->period > 0 && b->t % b->period == 0 && n >= b->period &&
-            build_graph(b)) {
-            if (cudaGraphLaunch(b->exec, b->stream) != cudaSuccess) return poison(b);
+            build_graph(b, b->cur)) {
+            if (cudaGraphLaunch(b->exec[b->cur], b->stream) != cudaSuccess) return poison(b);
             b->t += b->period;
-            n -= b->period;   // period is even: the buffers are back to 0
+            n -= b->period;
+            b->cur ^= b->period_flips;
         } else {
-            if (enqueue_step(b, b->stream, b->t, b->cur) != cudaSuccess) return poison(b);
-            b->t += 1;
+            int taken = 1;
+            if (enqueue_steps(b, b->stream, b->t, b->cur, n, taken) != cudaSuccess)
+                return poison(b);
+            b->t += taken;
             b->cur ^= 1;
-            n -= 1;
+            n -= taken;
         }
     }
     for (lb_state* s : b->reps) {

@@ -31,6 +31,8 @@
 #include "lb_packed.cuh"
 
 #include <type_traits>
+#include <utility>
+#include <vector>
 
 namespace lbsc {
 namespace {
@@ -545,7 +547,101 @@ cudaError_t launch_pair(const StepArgs<T>& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// The pairs of a batch: a persistent grid strides over a work list of tiles (replica,
+// first column, first row, end row) of every replica. The replica's arguments are
+// staged in shared memory by warp 0 when the replica changes.
+template <typename T, bool OM1, bool ODD>
+__global__ void __launch_bounds__(kTH, kPairThreads<T, OM1> / kTH)
+    k_step2_batch(const StepArgs<T>* __restrict__ args, const int4* __restrict__ tiles, int ntiles)
+{
+    __shared__ PairShared<T, kTH, OM1> sh;
+    __shared__ StepArgs<T> sa;
+    __shared__ PackedArgs sk;
+    __shared__ int sa_rep;
+    if (threadIdx.x == 0) sa_rep = -1;
+    for (int i = blockIdx.x; i < ntiles; i += gridDim.x) {
+        const int4 tl = __ldg(tiles + i);
+        __syncthreads();                            // previous tile done with the shared memory
+        if (threadIdx.x < 32 && tl.x != sa_rep) {
+            const int* src = reinterpret_cast<const int*>(args + tl.x);
+            int* dst = reinterpret_cast<int*>(&sa);
+            for (int w = threadIdx.x; w < (int)(sizeof(StepArgs<T>) / 4); w += 32)
+                dst[w] = __ldg(src + w);
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                sk = packed_args(sa);
+                sa_rep = tl.x;
+            }
+        }
+        __syncthreads();
+        const StepArgs<T> a = sa;
+        pair_tile<T, kTH, OM1, ODD>(a, sk, sh, tl.y, tl.z, tl.w);
+    }
+}
+
+template <typename T>
+cudaError_t launch_batch_pair(const BatchLaunch<T>& b, const int4* tiles, int ntiles, bool odd,
+                              cudaStream_t s)
+{
+    const int per_sm = (b.om1 ? kPairThreads<T, true> : kPairThreads<T, false>) / kTH;
+    const int grid = ntiles < per_sm * b.num_sms ? ntiles : per_sm * b.num_sms;
+    if (b.om1 && odd) k_step2_batch<T, true, true><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
+    else if (b.om1) k_step2_batch<T, true, false><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
+    else if (odd) k_step2_batch<T, false, true><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
+    else k_step2_batch<T, false, false><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
+    return cudaGetLastError();
+}
+
 }  // namespace
+
+// Work list of a batch's pair kernel. Chunk heights are balanced within a replica;
+// the height is the one that makes the estimated time least: waves of resident CTAs,
+// each as long as its tallest tile plus nine rows (the two half-busy ends of a tile
+// and its prologue).
+void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, bool om1, int num_sms,
+                std::vector<int4>& tiles)
+{
+    constexpr int W = 2 * kTH - 8;
+    const int threads = elem_bytes == 2 ? (om1 ? kPairThreads<__half, true> : kPairThreads<__half, false>)
+                                        : (om1 ? kPairThreads<float, true> : kPairThreads<float, false>);
+    const long long slots = (long long)(threads / kTH) * num_sms;
+    auto chunks_of = [](int ny, int rows) { return (ny + rows - 1) / rows; };
+    int tallest = 8;
+    for (const auto& s : sizes) tallest = s.second > tallest ? s.second : tallest;
+    int best = 8;
+    double best_cost = 1e30;
+    for (int rows = 8; rows <= tallest && rows <= 1024; ++rows) {
+        long long n = 0;
+        int high = 0;
+        for (const auto& s : sizes) {
+            const int c = chunks_of(s.second, rows), h = (s.second + c - 1) / c;
+            n += (long long)((s.first + W - 1) / W) * c;
+            high = h > high ? h : high;
+        }
+        const double cost = (double)((n + slots - 1) / slots) * (high + 9);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = rows;
+        }
+    }
+    for (size_t r = 0; r < sizes.size(); ++r) {
+        const int ny = sizes[r].second, c = chunks_of(ny, best), h = (ny + c - 1) / c;
+        for (int y = 0; y < ny; y += h)
+            for (int x = 0; x < sizes[r].first; x += W)
+                tiles.push_back(make_int4((int)r, x, y, y + h < ny ? y + h : ny));
+    }
+}
+
+cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int ntiles, bool odd,
+                            cudaStream_t s)
+{
+    return launch_batch_pair<float>(b, tiles, ntiles, odd, s);
+}
+cudaError_t fp16_batch_pair(const BatchLaunch<__half>& b, const int4* tiles, int ntiles, bool odd,
+                            cudaStream_t s)
+{
+    return launch_batch_pair<__half>(b, tiles, ntiles, odd, s);
+}
 
 cudaError_t fp32_step_pair(const StepArgs<float>& a, cudaStream_t s) { return launch_pair<float>(a, s); }
 cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s) { return launch_pair<__half>(a, s); }

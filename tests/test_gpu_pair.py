@@ -29,3 +29,28 @@ def test_paired_steps_equal_single_steps(nx, ny, prec, omega):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("sizes", [[(5, 5)], [(96, 80), (121, 33), (240, 17)],
+                                   [(64, 700), (5, 9), (1500, 12), (120, 120)]])
+@pytest.mark.parametrize("prec,omega", [("fp32", 1.0), ("fp32", 0.9), ("fp16_delta", 1.0),
+                                        ("fp16_delta", 1.2)])
+@pytest.mark.parametrize("trace", [0, 6, 20])
+def test_paired_batch_steps_equal_single_steps(sizes, prec, omega, trace):
+    """A batch stepped in one call (pairs, graph replay, odd numbers of buffer swaps per
+    period) against one step per call (no pairs), and two calls that split a period."""
+    from paper_1008_2865_gb300 import Batch, inputs
+    rhos = [inputs.noisy_density(nx, ny, seed=nx + ny, mean=0.7, amp=0.01, mode="rel")
+            for nx, ny in sizes]
+    om = [omega] + [1.0] * (len(sizes) - 1)
+    got = []
+    for chunks in ([1] * 47, [47], [3, 37, 7]):
+        with Batch(rhos, omega=om, G1=-5.0, G2=0.6, prec=prec, trace_every=trace) as b:
+            for n in chunks:
+                b.step(n)
+            got.append([(*b.fields(i), b.trace(i)) for i in range(len(b))])
+            assert b.t == 47
+    for other in got[1:]:
+        for one, two in zip(got[0], other):
+            for p, q in zip(one, two):
+                assert np.array_equal(p, q)
