@@ -100,6 +100,10 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
  * Eq. FORCE taken with the attractive sign of Eq. forza, BGK collision
  * towards the Eq. 4 equilibrium at the shifted velocity u + F/(omega rho),
  * then streaming. States t with t % trace_every == 0 append a trace row.
+ * Steps may share a launch: an FP32 or FP16 lattice that fits the SMs' shared memory
+ * (about 690 x 690 with omega = 1) takes all n in one cooperative launch, others two
+ * at a time; the results are those of single steps, bit for bit. In a stream capture
+ * every step is a launch of its own.
  * Asynchronous. Errors: LB_ERR_ARG (n < 0), LB_ERR_STATE, LB_ERR_CUDA. */
 lb_status lb_step(lb_state* s, long n);
 
@@ -141,8 +145,8 @@ lb_status lb_trace(lb_state* s, double* buf, int cap, int* count);
  * lb_init starts with pipeline 0 (measured the faster of the two on GB300 for
  * the 8192 x 8192 lattice). rows_per_cta is in
  * [4, 4096]. With pipeline 0 the shape is that of the steps taken one at a time
- * (those that append a trace row, and a last odd one); lb_step takes other steps
- * two at a time through a kernel with a shape of its own.
+ * and of the sums behind a trace row; steps that share a launch have shapes of
+ * their own.
  * The shape changes how the work is split, not the trajectory;
  * only the FP32 rounding of the energy partial sums depends on it.
  * Errors: LB_ERR_ARG for NULL or unsupported values, LB_ERR_STATE for an FP64
@@ -150,14 +154,16 @@ lb_status lb_trace(lb_state* s, double* buf, int cap, int* count);
 lb_status lb_get_launch(const lb_state* s, int* block_x, int* rows_per_cta, int* pipeline);
 lb_status lb_set_launch(lb_state* s, int block_x, int rows_per_cta, int pipeline);
 
-/* Bound on every in-kernel wait of the bulk-copy pipeline, in SM clock cycles
+/* Bound on every in-kernel wait (the bulk-copy pipeline's; a small lattice's tiles
+ * waiting for their neighbours' halo values), in SM clock cycles
  * (default 2e9, about one second at GB300 clocks). A wait that runs out makes
  * the kernel record an error and return; the next synchronising call
  * (lb_energy, lb_fields, lb_trace) reports LB_ERR_TIMEOUT and poisons the
  * state, while the CUDA context stays usable. test_skip_copies is a test hook
  * (0 or 1): with 1, every CTA arms the barrier of its first row unit for the
  * unit's bytes but issues none of the unit's copies, so that wait runs out on
- * purpose with nothing of the unit in flight; use 0 otherwise.
+ * purpose with nothing of the unit in flight, and the first tile of a small
+ * lattice marks its halo values with a step nobody waits for; use 0 otherwise.
  * Errors: LB_ERR_ARG (NULL, cycles <= 0, test_skip_copies not 0 or 1). */
 lb_status lb_set_wait_limit(lb_state* s, long long cycles, int test_skip_copies);
 

@@ -230,8 +230,38 @@ void free_state(lb_state* s)
     delete s;
 }
 
+// Steps of a small lattice that stay on the SMs (lb_resident.cu): from two steps on,
+// as many per launch as the trace rows they append can be kept.
+lb_status step_resident(lb_state* s, long n)
+{
+    ResidentBuf& b = s->res_buf;
+    while (n > 0) {
+        long m = n;
+        if (b.trace_every > 0) {
+            const long long te = b.trace_every;
+            const long long first = (s->t + te - 1) / te * te;   // next trace row
+            const long long room = first + te * b.max_rows - s->t;
+            if (m > room) m = (long)room;
+        }
+        if (m > (1L << 20)) m = 1L << 20;
+        const cudaError_t e =
+            s->p.prec == LB_FP32
+                ? fp32_resident(make_args<float>(s), b, s->launch.block_x, (int)m, s->stream)
+                : fp16_resident(make_args<__half>(s), b, s->launch.block_x, (int)m, s->stream);
+        if (e != cudaSuccess) return fail_cuda(s);
+        s->cur ^= 1;
+        s->t += m;
+        n -= m;
+    }
+    return LB_OK;
+}
+
 lb_status step_fp32(lb_state* s, long n)
 {
+    // in a stream capture every step is a launch of its own, so that a graph of an even
+    // number of steps can be replayed: each step swaps the buffers once
+    const bool many = n >= 2 && s->launch.pipeline == 0 && !stream_captures(s->stream);
+    if (many && s->res_buf.gx > 0) return step_resident(s, n);
     for (long k = 0; k < n; ++k) {
         const bool reduce = s->p.trace_every > 0 && (s->t % s->p.trace_every) == 0;
         cudaError_t e;
@@ -240,7 +270,7 @@ lb_status step_fp32(lb_state* s, long n)
         // (lb_pair.cu): the same fields bit for bit, half the memory traffic
         const bool next_reduces =
             s->p.trace_every > 0 && ((s->t + 1) % s->p.trace_every) == 0;
-        if (!bulk && !reduce && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
+        if (many && !reduce && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
             e = s->p.prec == LB_FP32 ? fp32_step_pair(make_args<float>(s), s->stream)
                                      : fp16_step_pair(make_args<__half>(s), s->stream);
             if (e != cudaSuccess) return fail_cuda(s);
@@ -314,6 +344,14 @@ const char* lb_status_str(lb_status st)
 lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, void* stream)
 {
     NvtxRange nvtx_range("lb_init");
+    return lbsc::state_init(out, p, rho_init, stream, true);
+}
+
+}  // extern "C"
+
+lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho_init, void* stream,
+                           bool alone)
+{
     if (!out) return LB_ERR_ARG;
     *out = nullptr;
     if (validate(p) != LB_OK || !rho_init) return LB_ERR_ARG;
@@ -359,6 +397,39 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
              alloc((void**)&s->dpsi[0], sizeof(float) * N) &&
              alloc((void**)&s->dpsi[1], sizeof(float) * N);
     }
+    ResidentBuf& rb = s->res_buf;
+    size_t word_bytes = 0;
+    if (ok && alone && p->prec != LB_FP64) {
+        int sms = 0;
+        const bool om1 = (float)p->omega == 1.0f;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
+            cudaGetLastError();
+            sms = 0;
+        }
+        if (resident_plan(p->nx, p->ny, om1, sms, rb)) {
+            rb.trace_every = p->trace_every;
+            word_bytes = resident_words(N, om1);
+            size_t bytes = word_bytes + 256;
+            // partials of one trace row: of the smallest CTAs a shape may have, and CTA rows
+            const size_t row_cap = (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0}) +
+                                   (size_t)s->max_cta_rows;
+            if (p->trace_every > 0) {
+                const long long rows = (8LL << 20) / (8 * N);
+                rb.max_rows = (int)(rows < 2 ? 2 : rows > 16 ? 16 : rows);
+                bytes += (size_t)rb.max_rows * (8 * (size_t)N + 4 * sizeof(double) * row_cap);
+            }
+            char* m = nullptr;
+            ok = alloc((void**)&m, bytes);
+            if (ok) {
+                // the words and counters first: they start cleared
+                rb.counters = reinterpret_cast<unsigned int*>(m);
+                rb.llm = reinterpret_cast<uint4*>(m + 256);
+                rb.llp = reinterpret_cast<uint2*>(rb.llm + (size_t)2 * (om1 ? 1 : 3) * N);
+                rb.partials = reinterpret_cast<double*>(m + 256 + word_bytes);
+                rb.dump = reinterpret_cast<float*>(rb.partials + (size_t)rb.max_rows * 4 * row_cap);
+            }
+        }
+    }
     if (!ok) {
         free_state(s);
         return LB_ERR_OOM;
@@ -378,7 +449,9 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
         cudaMemsetAsync(s->counter, 0, sizeof(unsigned int), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->trace_count, 0, sizeof(int), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess)
+        cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess ||
+        (rb.gx > 0 &&
+         cudaMemsetAsync(rb.counters, 0, 256 + word_bytes, s->stream) != cudaSuccess))
         return bail(LB_ERR_CUDA);
     if (rho_check_sum(rho_in, N, s->partials, s->counter, s->res, s->flag, s->stream) !=
         cudaSuccess)
@@ -420,6 +493,8 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
     *out = s;
     return LB_OK;
 }
+
+extern "C" {
 
 lb_status lb_step(lb_state* s, long n)
 {

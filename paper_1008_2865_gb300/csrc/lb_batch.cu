@@ -153,16 +153,16 @@ BatchLaunch<T> batch_launch(const lb_batch* b, int cur)
                           b->num_sms, b->alternate};
 }
 
-// Enqueue step t (buffers `cur` in) of every replica on stream s, or steps t and t + 1
-// together when `left` allows and neither appends a trace row; returns through `taken`
+// Enqueue step t (buffers `cur` in) of every replica on stream s, or (`pairs`) steps t and
+// t + 1 together when `left` allows and neither appends a trace row; returns through `taken`
 // how many steps that was. Either way the buffers swap once.
 cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cur, long long left,
-                          int& taken)
+                          bool pairs, int& taken)
 {
     const int te = b->trace_every;
     const bool reduce = te > 0 && t % te == 0;
     const bool next_reduces = te > 0 && (t + 1) % te == 0;
-    taken = !reduce && !next_reduces && left >= 2 ? 2 : 1;
+    taken = pairs && !reduce && !next_reduces && left >= 2 ? 2 : 1;
     if (b->prec == LB_FP32) {
         const BatchLaunch<float> L = batch_launch<float>(b, cur);
         return taken == 2 ? fp32_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, s)
@@ -185,7 +185,7 @@ bool build_graph(lb_batch* b, int cur)
     cudaError_t e = cudaSuccess;
     int in = cur;
     for (int k = 0, taken = 0; k < b->period && e == cudaSuccess; k += taken) {
-        e = enqueue_steps(b, b->cap, k, in, b->period - k, taken);
+        e = enqueue_steps(b, b->cap, k, in, b->period - k, true, taken);
         in ^= 1;
     }
     cudaGraph_t g = nullptr;
@@ -241,7 +241,7 @@ lb_status lb_batch_init(lb_batch** out, int count, const lb_params* params,
     b->trace_every = params[0].trace_every;
     for (int r = 0; r < count; ++r) {
         lb_state* s = nullptr;
-        const lb_status st = lb_init(&s, &params[r], rho_init[r], stream);
+        const lb_status st = state_init(&s, &params[r], rho_init[r], stream, false);
         if (st != LB_OK) {
             lb_batch_destroy(b);
             return st;
@@ -279,8 +279,10 @@ lb_status lb_batch_step(lb_batch* b, long n)
     if (b->poisoned) return LB_ERR_STATE;
     DeviceScope dev(b->device);
     if (!dev.ok) return poison(b);
+    // in a caller's capture every step is a launch of its own and swaps the buffers once
+    const bool captures = stream_captures(b->stream);
     while (n > 0) {
-        if (b->use_graph && b->period > 0 && b->t % b->period == 0 && n >= b->period &&
+        if (b->use_graph && !captures && b->period > 0 && b->t % b->period == 0 && n >= b->period &&
             build_graph(b, b->cur)) {
             if (cudaGraphLaunch(b->exec[b->cur], b->stream) != cudaSuccess) return poison(b);
             b->t += b->period;
@@ -288,7 +290,7 @@ lb_status lb_batch_step(lb_batch* b, long n)
             b->cur ^= b->period_flips;
         } else {
             int taken = 1;
-            if (enqueue_steps(b, b->stream, b->t, b->cur, n, taken) != cudaSuccess)
+            if (enqueue_steps(b, b->stream, b->t, b->cur, n, !captures, taken) != cudaSuccess)
                 return poison(b);
             b->t += taken;
             b->cur ^= 1;

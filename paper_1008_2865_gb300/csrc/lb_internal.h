@@ -51,6 +51,17 @@ struct DeviceScope {
     DeviceScope& operator=(const DeviceScope&) = delete;
 };
 
+// Whether the caller is capturing `s` into a graph.
+inline bool stream_captures(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 constexpr int kTraceCap = 65536;     // rows kept in the device trace ring
 constexpr int kTraceCols = 5;        // (t, mass, E_s, E_m, E_bulk)
 
@@ -162,9 +173,10 @@ struct BatchLaunch {
 };
 cudaError_t fp32_batch_step(const BatchLaunch<float>& b, bool reduce, cudaStream_t s);
 cudaError_t fp16_batch_step(const BatchLaunch<__half>& b, bool reduce, cudaStream_t s);
-// Two plain steps in one pass (lb_pair.cu), for lattices of 2^18 sites on: below, its
-// few long chunks take as long as two launches of k_step (us per step, single and
-// paired: 250x187 10.1 and 10.2, 512^2 10.3 and 9.3, 700^2 12.3 and 10.2).
+// Two plain steps in one pass (lb_pair.cu), for lattices of 2^18 sites on that are not
+// held on the SMs (lb_resident.cu): below, its few long chunks take as long as two
+// launches of k_step (us per step, single and paired: 250x187 10.1 and 10.2, 512^2 10.3
+// and 9.3, 700^2 12.3 and 10.2).
 inline bool pairs_pay(long long n) { return n >= (1LL << 18); }
 cudaError_t fp32_step_pair(const StepArgs<float>& a, cudaStream_t s);
 cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s);
@@ -178,6 +190,25 @@ cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int 
                             cudaStream_t s);
 cudaError_t fp16_batch_pair(const BatchLaunch<__half>& b, const int4* tiles, int ntiles, bool odd,
                             cudaStream_t s);
+// Many steps of a small lattice in one launch (lb_resident.cu): the tiles its CTAs hold
+// and the buffers they exchange through.
+struct ResidentBuf {
+    int gx = 0, gy = 0, tw = 0, th = 0;   // tile grid and tile size; gx = 0: not used
+    unsigned tag = 0;                     // steps exchanged so far
+    uint2* llp = nullptr;                 // halo words of dpsi
+    uint4* llm = nullptr;                 // halo words of the moments or populations
+    int trace_every = 0;
+    int max_rows = 0;                     // trace rows one launch may dump
+    float* dump = nullptr;                // [max_rows][2][N]
+    double* partials = nullptr;           // [max_rows][partials of one trace row][4]
+    unsigned int* counters = nullptr;     // [1 + max_rows]
+};
+bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b);
+size_t resident_words(long long n, bool om1);   // bytes of the halo words
+cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps,
+                          cudaStream_t s);
+cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps,
+                          cudaStream_t s);
 // bulk-copy pipelined step (lb_bulk.cu)
 bool bulk_supported(int nx, int ny, int elem_bytes, int block_x);
 int bulk_grid_blocks(int nx, int ny, int elem_bytes, Fp32Launch L);
@@ -236,6 +267,7 @@ struct lb_state {
     int* err = nullptr;            // set by a kernel whose bounded wait ran out
     long long wait_cycles = 2000000000LL;
     int skip_unit0 = 0;            // test hook of lb_set_wait_limit
+    lbsc::ResidentBuf res_buf;     // small lattices: tiles held on the SMs over many steps
     // FP64 parity storage
     double* f64[2] = {nullptr, nullptr};
     double* psi64 = nullptr;
@@ -259,6 +291,9 @@ struct lb_state {
 };
 
 namespace lbsc {
+// lb_init; `alone`: the state is stepped by itself (false for a batch's replicas)
+lb_status state_init(lb_state** out, const lb_params* p, const double* rho_init, void* stream,
+                     bool alone);
 constexpr size_t kGuardBytes = 256;              // guard region on each side of a buffer
 constexpr unsigned char kGuardByte = 0xA5;       // the pattern the guards hold
 // Allocate `bytes` for a state with guards on both sides (pattern written on
