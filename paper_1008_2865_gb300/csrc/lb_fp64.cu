@@ -14,7 +14,13 @@
 // With identical order and correctly rounded exp, the result of each step is
 // fixed bit for bit by these definitions, so any other evaluation that
 // follows them reproduces it exactly. The state is f(t) after streaming.
-// This path is for verification; it is not tuned.
+// The path is bound by FP64 instructions (a slow pipe on this part), so no operation is
+// spent that cannot change a bit: products with the lattice vectors' 0 and +-1 are not
+// formed (site_plain keeps them for states that are no longer finite), and exp is first
+// evaluated to 2^-78 and only then, if that leaves the rounding open, to the last bit.
+// 128^2: 96 -> 18.5 us per step; 1024^2 610 us, where the 310 FP64 operations of a site
+// are the bound (two per clock and SM).
+#include "lb_exp_table.h"
 #include "lb_internal.h"
 
 namespace lbsc {
@@ -94,7 +100,7 @@ __host__ __device__ __forceinline__ dd dd_div_d(dd a, double b)
     return quick_two_sum(q1, q2);
 }
 
-__host__ __device__ double exp_cr(double x)
+__device__ __noinline__ double exp_cr(double x)
 {
     // ln 2 = LN2_HI + LN2_LO to ~2^-107 (the two leading double parts of ln 2)
     const double LN2_HI = 6.93147180559945286227e-01;
@@ -118,6 +124,43 @@ __host__ __device__ double exp_cr(double x)
     const dd e = dd_add_d(m, 1.0);
     const double v = e.hi + e.lo;     // the one rounding to double
     return ldexp(v, (int)k);
+}
+
+// The same result, usually after some 50 instead of 2000 FP64 operations: x = (256 m + j)
+// ln2/256 + r with |r| <= ln2/512, e^x = 2^m 2^(j/256) e^r, the table and r in two
+// doubles each and e^r - 1 by its series, whose terms from r^3 on are below 2^-31 and
+// need one double only. The relative error of v + lo is below 2^-81 for |x| < 32 (sum of
+// the terms' bounds: 2^-83 for ln2/256, 2^-82 for the series' double part, 2^-83 for the
+// sums; 2^-81.96 the largest of 30,000 samples against 400-bit arithmetic). If adding
+// 2^-78 either way rounds alike, that is the correctly rounded value; otherwise (about
+// once in 2^24) exp_cr decides. (Rounding test: Ziv, "Fast evaluation of elementary
+// mathematical functions with correctly rounded last bit", 1991.)
+__device__ __forceinline__ double exp_rounded(double x)
+{
+    if (fabs(x) < 32.0) {
+        // ln 2 / 256 = L1 + L2, L1 of 35 bits so that k L1 is exact
+        const double L1 = 0x1.62e42fefcp-9, L2 = -0x1.c610ca86c3899p-45;
+        const double k = rint(x * 0x1.71547652b82fep+8);
+        const dd r = two_sum(fma(-k, L1, x), -(k * L2));
+        const dd r2 = two_prod(r.hi, r.hi);
+        const double r2lo = fma(2.0 * r.hi, r.lo, r2.lo);
+        double q = fma(r.hi, 1.0 / 5040.0, 1.0 / 720.0);
+        q = fma(r.hi, q, 1.0 / 120.0);
+        q = fma(r.hi, q, 1.0 / 24.0);
+        q = fma(r.hi, q, 1.0 / 6.0);
+        q = (r.hi * r2.hi) * q;
+        const dd s = two_sum(r.hi, 0.5 * r2.hi);
+        const dd e = quick_two_sum(s.hi, ((s.lo + r.lo) + 0.5 * r2lo) + q);
+        const int ki = (int)k;
+        const double2 t = __ldg(&kExp2Table[ki & 255]);
+        const dd p = two_prod(t.x, e.hi);
+        const dd v = two_sum(t.x, p.hi);
+        const double lo = v.lo + (p.lo + (fma(t.x, e.lo, t.y) + t.y * e.hi));
+        const double eps = 0x1p-78 * v.hi;
+        const double up = v.hi + (lo + eps), dn = v.hi + (lo - eps);
+        if (up == dn) return up * __longlong_as_double((long long)((ki >> 8) + 1023) << 52);
+    }
+    return exp_cr(x);
 }
 
 // ---------------------------------------------------------------- lattice
@@ -174,58 +217,159 @@ __global__ void k64_psi(const Fp64Args a)
     const double sq = sqrt(a.rho0);
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N;
          s += (long long)gridDim.x * blockDim.x) {
-        double r, jx, jy;
-        moments(a.f_in, N, s, r, jx, jy);
+        double r = 0.0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) r = r + a.f_in[i * N + s];
         a.rho[s] = r;
-        a.psi[s] = sq * (1.0 - exp_cr(-r / a.rho0));
+        const double x = a.rho0 == 1.0 ? -r : -r / a.rho0;
+        a.psi[s] = sq * (1.0 - exp_rounded(x));
     }
 }
 
+// Collision and streaming of one site with every product formed: for sites whose
+// density or force is not finite, where a dropped 0 * inf would show.
+__device__ __noinline__ void site_plain(const Fp64Args& a, long long s, int x, int y)
+{
+    const int nx = a.nx, ny = a.ny;
+    const long long N = (long long)nx * ny;
+    const double om = a.omega;
+    double rho, jx, jy;
+    moments(a.f_in, N, s, rho, jx, jy);
+    double wx = 0.0, wy = 0.0, sx = 0.0, sy = 0.0, mx = 0.0, my = 0.0;
+    for (int i = 1; i <= 8; ++i) {
+        const double pn = a.psi[site(x + CX[i], y + CY[i], nx, ny)];
+        wx = wx + (W[i] * pn) * (double)CX[i];
+        wy = wy + (W[i] * pn) * (double)CY[i];
+        sx = sx + (PS[i] * pn) * (double)CX[i];
+        sy = sy + (PS[i] * pn) * (double)CY[i];
+    }
+    for (int k = 0; k < 16; ++k) {
+        const double pn = a.psi[site(x + MX[k], y + MY[k], nx, ny)];
+        mx = mx + (PM[k] * pn) * (double)MX[k];
+        my = my + (PM[k] * pn) * (double)MY[k];
+    }
+    const double ps = a.psi[s];
+    const double Fsx = (a.G1 * ps) * wx + (a.G2 * ps) * sx;
+    const double Fsy = (a.G1 * ps) * wy + (a.G2 * ps) * sy;
+    const double Fmx = (a.G2 * ps) * mx;
+    const double Fmy = (a.G2 * ps) * my;
+    const double Fx = -(Fsx + Fmx);
+    const double Fy = -(Fsy + Fmy);
+    const double ux = jx / rho;
+    const double uy = jy / rho;
+    const double orho = om * rho;
+    const double vx = ux + Fx / orho;
+    const double vy = uy + Fy / orho;
+    const double usq = vx * vx + vy * vy;
+    for (int i = 0; i < 9; ++i) {
+        const double cu = (double)CX[i] * vx + (double)CY[i] * vy;
+        const double feq = (W[i] * rho) * (((1.0 + 3.0 * cu) + (4.5 * cu) * cu) - 1.5 * usq);
+        const double fi = a.f_in[i * N + s];
+        a.f_out[i * N + site(x + CX[i], y + CY[i], nx, ny)] = fi - om * (fi - feq);
+    }
+}
+
+// The periodic neighbourhood of a site (nx, ny >= 5): columns x-2 .. x+2, row offsets.
+struct Nbr {
+    int x[5];
+    long long y[5];
+};
+__device__ __forceinline__ Nbr neighbours(int x, int y, int nx, int ny)
+{
+    Nbr n;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        int xx = x + k - 2, yy = y + k - 2;
+        xx += xx < 0 ? nx : 0;
+        xx -= xx >= nx ? nx : 0;
+        yy += yy < 0 ? ny : 0;
+        yy -= yy >= ny ? ny : 0;
+        n.x[k] = xx;
+        n.y[k] = (long long)yy * nx;
+    }
+    return n;
+}
+
+// One site per thread, in the order of site_plain without the products that cannot
+// change a finite result: a term with c = 0 adds a zero, c = +-1 a sign, c = +-2 is exact
+// (so a fused multiply-add with it rounds once, as the addition would).
 __global__ void k64_collide_stream(const Fp64Args a)
 {
+    constexpr double w0 = 4.0 / 9.0, w1 = 1.0 / 9.0, w2 = 1.0 / 36.0;
+    constexpr double p1 = 4.0 / 63.0, p2 = 4.0 / 135.0, p4 = 1.0 / 180.0, p5 = 2.0 / 945.0,
+                     p8 = 1.0 / 15120.0;
     const int nx = a.nx, ny = a.ny;
     const long long N = (long long)nx * ny;
     const double om = a.omega;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N;
          s += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(s / nx), x = (int)(s % nx);
-        double rho, jx, jy;
-        moments(a.f_in, N, s, rho, jx, jy);
-        double wx = 0.0, wy = 0.0, sx = 0.0, sy = 0.0, mx = 0.0, my = 0.0;
+        const int y = (int)(s / nx), x = (int)(s - (long long)y * nx);
+        const Nbr nb = neighbours(x, y, nx, ny);
+        double f[9];
 #pragma unroll
-        for (int i = 1; i <= 8; ++i) {
-            const double pn = a.psi[site(x + CX[i], y + CY[i], nx, ny)];
-            wx = wx + (W[i] * pn) * (double)CX[i];
-            wy = wy + (W[i] * pn) * (double)CY[i];
-            sx = sx + (PS[i] * pn) * (double)CX[i];
-            sy = sy + (PS[i] * pn) * (double)CY[i];
-        }
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const double pn = a.psi[site(x + MX[k], y + MY[k], nx, ny)];
-            mx = mx + (PM[k] * pn) * (double)MX[k];
-            my = my + (PM[k] * pn) * (double)MY[k];
-        }
+        for (int i = 0; i < 9; ++i) f[i] = a.f_in[i * N + s];
+        auto psi = [&](int dx, int dy) { return a.psi[nb.y[2 + dy] + nb.x[2 + dx]]; };
+        const double rho = ((((((((f[0] + f[1]) + f[2]) + f[3]) + f[4]) + f[5]) + f[6]) + f[7]) + f[8]);
+        const double jx = ((((f[1] - f[3]) + f[5]) - f[6]) - f[7]) + f[8];
+        const double jy = ((((f[2] - f[4]) + f[5]) + f[6]) - f[7]) - f[8];
+        // belt 1 in the D2Q9 order, with the w_i and the p_si
+        const double a1 = psi(1, 0), a2 = psi(0, 1), a3 = psi(-1, 0), a4 = psi(0, -1);
+        const double a5 = psi(1, 1), a6 = psi(-1, 1), a7 = psi(-1, -1), a8 = psi(1, -1);
+        auto belt1 = [&](double u, double d, double& bx, double& by) {
+            const double q5 = d * a5, q6 = d * a6, q7 = d * a7, q8 = d * a8;
+            bx = ((((u * a1 - u * a3) + q5) - q6) - q7) + q8;
+            by = ((((u * a2 - u * a4) + q5) + q6) - q7) - q8;
+        };
+        double wx, wy, sx, sy;
+        belt1(w1, w2, wx, wy);
+        belt1(p1, p2, sx, sy);
+        // belt 2 in the order of Table 1
+        double mx = 2.0 * (p4 * psi(2, 0)), my = 2.0 * (p4 * psi(0, 2));
+        mx = fma(-2.0, p4 * psi(-2, 0), mx);
+        my = fma(-2.0, p4 * psi(0, -2), my);
+        auto link = [&](double p, int cx, int cy) {
+            const double q = p * psi(cx, cy);
+            mx = cx == 1 ? mx + q : cx == -1 ? mx - q : fma((double)cx, q, mx);
+            my = cy == 1 ? my + q : cy == -1 ? my - q : fma((double)cy, q, my);
+        };
+        link(p5, 2, 1);
+        link(p5, 1, 2);
+        link(p5, -1, 2);
+        link(p5, -2, 1);
+        link(p5, -2, -1);
+        link(p5, -1, -2);
+        link(p5, 1, -2);
+        link(p5, 2, -1);
+        link(p8, 2, 2);
+        link(p8, -2, 2);
+        link(p8, -2, -2);
+        link(p8, 2, -2);
         const double ps = a.psi[s];
-        const double Fsx = (a.G1 * ps) * wx + (a.G2 * ps) * sx;
-        const double Fsy = (a.G1 * ps) * wy + (a.G2 * ps) * sy;
-        const double Fmx = (a.G2 * ps) * mx;
-        const double Fmy = (a.G2 * ps) * my;
-        const double Fx = -(Fsx + Fmx);
-        const double Fy = -(Fsy + Fmy);
-        const double ux = jx / rho;
-        const double uy = jy / rho;
+        const double g1p = a.G1 * ps, g2p = a.G2 * ps;
+        const double Fx = -((g1p * wx + g2p * sx) + g2p * mx);
+        const double Fy = -((g1p * wy + g2p * sy) + g2p * my);
         const double orho = om * rho;
-        const double vx = ux + Fx / orho;
-        const double vy = uy + Fy / orho;
-        const double usq = vx * vx + vy * vy;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const double cu = (double)CX[i] * vx + (double)CY[i] * vy;
-            const double feq = (W[i] * rho) * (((1.0 + 3.0 * cu) + (4.5 * cu) * cu) - 1.5 * usq);
-            const double fi = a.f_in[i * N + s];
-            a.f_out[i * N + site(x + CX[i], y + CY[i], nx, ny)] = fi - om * (fi - feq);
+        const double vx = jx / rho + Fx / orho;
+        const double vy = jy / rho + Fy / orho;
+        if (!(isfinite(rho) && isfinite(Fx) && isfinite(Fy) && isfinite(vx) && isfinite(vy))) {
+            site_plain(a, s, x, y);
+            continue;
         }
+        const double u15 = 1.5 * (vx * vx + vy * vy);
+        auto put = [&](int i, int cx, int cy, double feq) {
+            a.f_out[i * N + nb.y[2 + cy] + nb.x[2 + cx]] = f[i] - om * (f[i] - feq);
+        };
+        put(0, 0, 0, (w0 * rho) * (1.0 - u15));
+        auto axis = [&](int i, int j, int cx, int cy, double wr, double cu) {
+            const double t = 3.0 * cu, q = (4.5 * cu) * cu;
+            put(i, cx, cy, wr * (((1.0 + t) + q) - u15));
+            put(j, -cx, -cy, wr * (((1.0 - t) + q) - u15));
+        };
+        const double r1 = w1 * rho, r2 = w2 * rho;
+        axis(1, 3, 1, 0, r1, vx);
+        axis(2, 4, 0, 1, r1, vy);
+        axis(5, 7, 1, 1, r2, vx + vy);
+        axis(6, 8, -1, 1, r2, vy - vx);
     }
 }
 
@@ -262,22 +406,48 @@ __global__ void __launch_bounds__(256) k64_energy(const Fp64Args a, double* part
 {
     const int nx = a.nx, ny = a.ny;
     const long long N = (long long)nx * ny;
-    // rest weight of the E(8) set from Eq. weights_1
-    double p0 = 0.0;
-    for (int i = 1; i <= 8; ++i) p0 = p0 + PS[i];
-    for (int k = 0; k < 16; ++k) p0 = p0 + PM[k];
-    p0 = 1.0 - p0;
+    // the links' couplings G1 w_i + G2 p_si and G2 p_mi, the rest weight of the E(8) set
+    // from Eq. weights_1 summed link by link
+    constexpr double p1 = 4.0 / 63.0, p2 = 4.0 / 135.0, p4 = 1.0 / 180.0, p5 = 2.0 / 945.0,
+                     p8 = 1.0 / 15120.0;
+    constexpr double belt1 = p1 + p1 + p1 + p1 + p2 + p2 + p2 + p2;
+    constexpr double p0 = 1.0 - (belt1 + p4 + p4 + p4 + p4 + p5 + p5 + p5 + p5 + p5 + p5 + p5 + p5 +
+                                 p8 + p8 + p8 + p8);
+    const double k0 = a.G1 * (4.0 / 9.0) + a.G2 * p0, k1 = a.G1 * (1.0 / 9.0) + a.G2 * p1,
+                 k2 = a.G1 * (1.0 / 36.0) + a.G2 * p2;
+    const double k4 = a.G2 * p4, k5 = a.G2 * p5, k8 = a.G2 * p8;
     const double A1 = a.G1 + a.G2;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (long long s = blockIdx.x * 256LL + threadIdx.x; s < N; s += (long long)gridDim.x * 256) {
-        const int y = (int)(s / nx), x = (int)(s % nx);
+        const int y = (int)(s / nx), x = (int)(s - (long long)y * nx);
+        const Nbr nb = neighbours(x, y, nx, ny);
+        auto psi = [&](int dx, int dy) { return a.psi[nb.y[2 + dy] + nb.x[2 + dx]]; };
         const double ps = a.psi[s];
-        double ss = (a.G1 * W[0] + a.G2 * p0) * ps;
-        for (int i = 1; i <= 8; ++i)
-            ss = ss + (a.G1 * W[i] + a.G2 * PS[i]) * a.psi[site(x + CX[i], y + CY[i], nx, ny)];
-        double sm = 0.0;
-        for (int k = 0; k < 16; ++k)
-            sm = sm + (a.G2 * PM[k]) * a.psi[site(x + MX[k], y + MY[k], nx, ny)];
+        double ss = k0 * ps;
+        ss = ss + k1 * psi(1, 0);
+        ss = ss + k1 * psi(0, 1);
+        ss = ss + k1 * psi(-1, 0);
+        ss = ss + k1 * psi(0, -1);
+        ss = ss + k2 * psi(1, 1);
+        ss = ss + k2 * psi(-1, 1);
+        ss = ss + k2 * psi(-1, -1);
+        ss = ss + k2 * psi(1, -1);
+        double sm = k4 * psi(2, 0);
+        sm = sm + k4 * psi(0, 2);
+        sm = sm + k4 * psi(-2, 0);
+        sm = sm + k4 * psi(0, -2);
+        sm = sm + k5 * psi(2, 1);
+        sm = sm + k5 * psi(1, 2);
+        sm = sm + k5 * psi(-1, 2);
+        sm = sm + k5 * psi(-2, 1);
+        sm = sm + k5 * psi(-2, -1);
+        sm = sm + k5 * psi(-1, -2);
+        sm = sm + k5 * psi(1, -2);
+        sm = sm + k5 * psi(2, -1);
+        sm = sm + k8 * psi(2, 2);
+        sm = sm + k8 * psi(-2, 2);
+        sm = sm + k8 * psi(-2, -2);
+        sm = sm + k8 * psi(2, -2);
         v[0] = v[0] + (0.5 * ps) * ss;
         v[1] = v[1] + (0.5 * ps) * sm;
         v[2] = v[2] + ((0.5 * A1) * ps) * ps;
@@ -335,13 +505,18 @@ __global__ void k64_exp(const double* __restrict__ x, double* __restrict__ y, lo
         y[s] = exp_cr(x[s]);
 }
 
-int grid_for(long long n)
+int grid_for(long long n, int threads = 256)
 {
-    long long b = (n + 255) / 256;
-    if (b > 152 * 8) b = 152 * 8;
+    long long b = (n + threads - 1) / threads;
+    if (b > 152 * 2048 / threads) b = 152 * 2048 / threads;
     if (b < 1) b = 1;
     return (int)b;
 }
+
+// Threads per CTA of the step's kernels: small CTAs while the lattice has few sites per
+// SM, so that they spread evenly over the SMs' FP64 units (128^2 in CTAs of 256 fills
+// 64 of 152 SMs).
+int step_threads(long long n) { return n < 152LL * 1024 ? 32 : 128; }
 
 }  // namespace
 
@@ -353,13 +528,17 @@ cudaError_t fp64_init(double* f, const double* rho_init, int nx, int ny, cudaStr
 
 cudaError_t fp64_psi(const Fp64Args& a, cudaStream_t s)
 {
-    k64_psi<<<grid_for((long long)a.nx * a.ny), 256, 0, s>>>(a);
+    const long long n = (long long)a.nx * a.ny;
+    const int nt = step_threads(n);
+    k64_psi<<<grid_for(n, nt), nt, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t fp64_collide_stream(const Fp64Args& a, cudaStream_t s)
 {
-    k64_collide_stream<<<grid_for((long long)a.nx * a.ny), 256, 0, s>>>(a);
+    const long long n = (long long)a.nx * a.ny;
+    const int nt = step_threads(n);
+    k64_collide_stream<<<grid_for(n, nt), nt, 0, s>>>(a);
     return cudaGetLastError();
 }
 
