@@ -231,17 +231,22 @@ __device__ void accumulate_grid2(float v0, float v1, const AdjArgs& A)
     }
 }
 
-// J of the state (A.g / gT, A.dpsi) and the terminal adjoint l(T) (skipped when
-// A.lam is null: lb_objective). T is the population storage type.
-template <typename T>
+// J of the state (gT, A.dpsi) and, with GRAD, the terminal adjoint l(T) and the explicit
+// dE/dG1, dE/dG2 (lb_objective takes J alone; its sums are the same additions). T is the
+// population storage type. Rows of CTAs' sites are read as in k_delta_energy; a thread's
+// sums of psi times a class sum are exact FP32 products in two FP32 values (Two), the
+// misfit, whose target is FP64, is summed in FP64.
+template <typename T, bool GRAD>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_terminal(const AdjArgs A,
                                                               const T* __restrict__ gT)
 {
     const StepArgs<float>& a = A.a;
     const int nx = a.nx, ny = a.ny, N = (int)a.N;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};   // E, misfit, dE/dG1, dE/dG2
+    Two e{0.f, 0.f}, e1{0.f, 0.f}, e2{0.f, 0.f};
+    double mis2 = 0.0;
     for (int s = blockIdx.x * kAdjThreads + threadIdx.x; s < N; s += gridDim.x * kAdjThreads) {
-        const int y = s / nx, x = s % nx;
+        const int y = s / nx, x = s - y * nx;
+        const double target = __ldg(A.rho_target + s);
         float f[9];
         site_f(gT, a.pitch, x, y, f);
         const float d = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
@@ -260,21 +265,27 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_terminal(const AdjArgs A,
                                            ((p[4][3] + p[4][1]) + (p[0][3] + p[0][1])));
         const float S8 = fmaf(4.f, pr, (p[4][4] + p[4][0]) + (p[0][4] + p[0][0]));
         const float dEdpsi = a.K0 * pc + a.K1 * S1 + a.K2 * S2 + a.K4 * S4 + a.K5 * S5 + a.K8 * S8;
-        const float sw = A.aw.K0 * pc + A.aw.K1 * S1 + A.aw.K2 * S2;
-        const float sp = A.ap.K0 * pc + A.ap.K1 * S1 + A.ap.K2 * S2 + A.ap.K4 * S4 +
-                         A.ap.K5 * S5 + A.ap.K8 * S8;
-        const float dpr = __expf(-rho * a.inv_rho0) * A.inv_sqrt_rho0;
-        const double mis = (double)rho - A.rho_target[s];
-        if (A.lam) {
+        const double mis = (double)rho - target;
+        auto add_product = [&](Two& sum, float u, float v) {
+            const float q = __fmul_rn(u, v);
+            two_add(sum, q, __fmaf_rn(u, v, -q));
+        };
+        add_product(e, pc, dEdpsi);
+        mis2 += mis * mis;
+        if (GRAD) {
+            const float sw = A.aw.K0 * pc + A.aw.K1 * S1 + A.aw.K2 * S2;
+            const float sp = A.ap.K0 * pc + A.ap.K1 * S1 + A.ap.K2 * S2 + A.ap.K4 * S4 +
+                             A.ap.K5 * S5 + A.ap.K8 * S8;
+            const float dpr = __expf(-rho * a.inv_rho0) * A.inv_sqrt_rho0;
             const float lam = dpr * dEdpsi + (float)(2.0 * mis);
 #pragma unroll
             for (int i = 0; i < 9; ++i) A.lam[i * N + s] = lam;
+            add_product(e1, pc, sw);
+            add_product(e2, pc, sp);
         }
-        v[0] += 0.5 * (double)pc * dEdpsi;
-        v[1] += mis * mis;
-        v[2] += 0.5 * (double)pc * sw;
-        v[3] += 0.5 * (double)pc * sp;
     }
+    // E, misfit, dE/dG1, dE/dG2
+    double v[4] = {0.5 * value(e), mis2, 0.5 * value(e1), 0.5 * value(e2)};
     accumulate_grid<kAdjThreads>(v, A);
 }
 
@@ -530,7 +541,7 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
     A.dpsi = s->dpsi[s->cur];
     A.lam = lamA;
     A.acc = acc;             // acc[0..3] = E, misfit, dE/dG1, dE/dG2
-    k_adj_terminal<float><<<grid, kAdjThreads, 0, st>>>(A, A.g);
+    k_adj_terminal<float, true><<<grid, kAdjThreads, 0, st>>>(A, A.g);
     if (cudaGetLastError() != cudaSuccess) return fail();
 
     // ---- reverse over the segments. Segment k (states kC .. kC + n - 1) is
@@ -635,14 +646,13 @@ cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, c
     A.partials = s->partials;
     A.counter = s->counter;
     A.acc = acc;
-    A.lam = nullptr;
     cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const int grid = adj_grid(s->N);
     if (s->p.prec == LB_FP16_DELTA)
-        k_adj_terminal<__half><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const __half*>(s->g[s->cur]));
+        k_adj_terminal<__half, false><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const __half*>(s->g[s->cur]));
     else
-        k_adj_terminal<float><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const float*>(s->g[s->cur]));
+        k_adj_terminal<float, false><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const float*>(s->g[s->cur]));
     return cudaGetLastError();
 }
 

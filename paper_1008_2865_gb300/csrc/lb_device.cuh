@@ -286,6 +286,38 @@ __device__ __forceinline__ float dpsi_of(float d, const StepArgs<T>& a)
     return a.cpsi * expm1f(-d * a.inv_rho0);
 }
 
+// Unevaluated sums hi + lo of two FP32 values: products and sums of FP32 terms to about
+// 2^-46 of their magnitude on the FP32 pipe, where FP64 (64 times slower on this part)
+// would bound a kernel that streams memory (TwoSum: Knuth; TwoProduct with a fused
+// multiply-add: Ogita, Rump and Oishi, "Accurate sum and dot product", 2005). None of
+// the operations may be contracted or reassociated.
+struct Two {
+    float hi, lo;
+};
+// s += p exactly in the high part, the rounding errors and q in the low one
+__device__ __forceinline__ void two_add(Two& s, float p, float q)
+{
+    const float t = __fadd_rn(s.hi, p);
+    const float b = __fsub_rn(t, s.hi);
+    const float e = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, b)), __fsub_rn(p, b));
+    s.hi = t;
+    s.lo = __fadd_rn(s.lo, __fadd_rn(e, q));
+}
+// s += k x
+__device__ __forceinline__ void two_fma(Two& s, Two k, float x)
+{
+    const float p = __fmul_rn(k.hi, x);
+    two_add(s, p, __fmaf_rn(k.lo, x, __fmaf_rn(k.hi, x, -p)));
+}
+// s += a b
+__device__ __forceinline__ void two_fma(Two& s, Two a, Two b)
+{
+    const float p = __fmul_rn(a.hi, b.hi);
+    const float e = __fmaf_rn(a.hi, b.hi, -p);
+    two_add(s, p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e)));
+}
+__device__ __forceinline__ double value(Two s) { return (double)s.hi + (double)s.lo; }
+
 // Deterministic sum of 4 doubles over a CTA of NT threads (NT a multiple of
 // 32, at most 1024); the result is valid in thread 0. The threads' values meet
 // in shared memory and warp 0 alone does the FP64 adds (fixed strided order,

@@ -471,62 +471,77 @@ __global__ void __launch_bounds__(256) k_delta_fields(const T* __restrict__ g, i
     }
 }
 
+// The couplings of k_delta_energy, formed in FP64 on the host: E_s and E_m of a site are
+// psi/2 times cs + sum K S and cm + sum K S over the class sums S of the deviations.
+struct EnergyArgs {
+    Two K0, K1, K2, K4, K5, K8;
+    Two cs, cm;      // psi_ref (4 K1 + 4 K2), psi_ref (4 K4 + 8 K5 + 4 K8)
+};
+
 // lb_energy: the Sec. 5 sums and the mass of state t. Row by row (blockIdx.y
 // strides over rows, the threads of a block over columns; a column away from
 // the periodic x edges reads its stencil rows with immediate offsets). The
 // class sums of the psi deviations (|c|^2 = 1, 2, 4, 5, 8) and the site's
 // deviation sum are FP32 sums of 4-9 FP32 values (within a few units of
-// 2^-24 of their magnitude, ~1e-9 here); the products with the couplings and
-// every accumulation are FP64.
+// 2^-24 of their magnitude, ~1e-9 here); the products with the couplings and a
+// thread's sums are carried in two FP32 values each (Two), everything above a
+// thread in FP64. (4096^2, the whole call: 827 us with those in FP64, which then bounds the
+// kernel, 25 operations a site at two per clock and SM, 250 us now; the energies differ
+// by less than 1e-15 of their magnitude.)
 template <typename T>
 __global__ void __launch_bounds__(256) k_delta_energy(const T* __restrict__ g,
                                                       const float* __restrict__ dpsi,
-                                                      const StepArgs<T> a, double* out4)
+                                                      const StepArgs<T> a, const EnergyArgs k,
+                                                      double* out4)
 {
     const int nx = a.nx, ny = a.ny;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    const double pr = a.psi_ref;
-    const double K0 = a.K0, K1 = a.K1, K2 = a.K2, K4 = a.K4, K5 = a.K5, K8 = a.K8;
+    Two es{0.f, 0.f}, em{0.f, 0.f}, eb{0.f, 0.f}, ms{0.f, 0.f};
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
         const float* rw[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) rw[k] = dpsi + (size_t)wrapi(y + k - 2, ny) * nx;
+        for (int j = 0; j < 5; ++j) rw[j] = dpsi + (size_t)wrapi(y + j - 2, ny) * nx;
         for (int x = blockIdx.x * 256 + threadIdx.x; x < nx; x += gridDim.x * 256) {
-            float q[5][5];          // q[k][m] = dpsi(x + m - 2, y + k - 2)
+            float q[5][5];          // q[j][m] = dpsi(x + m - 2, y + j - 2)
             if (x >= 2 && x < nx - 2) {
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
+                for (int j = 0; j < 5; ++j) {
 #pragma unroll
-                    for (int m = 0; m < 5; ++m) q[k][m] = __ldg(rw[k] + x + m - 2);
+                    for (int m = 0; m < 5; ++m) q[j][m] = __ldg(rw[j] + x + m - 2);
                 }
             } else {
 #pragma unroll
                 for (int m = 0; m < 5; ++m) {
                     const int xx = wrapi(x + m - 2, nx);
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) q[k][m] = __ldg(rw[k] + xx);
+                    for (int j = 0; j < 5; ++j) q[j][m] = __ldg(rw[j] + xx);
                 }
             }
+            float f[9];
+            load_site_xy(f, g, a.pitch, x, y);
             const float S1 = (q[2][3] + q[2][1]) + (q[3][2] + q[1][2]);
             const float S2 = (q[3][3] + q[3][1]) + (q[1][3] + q[1][1]);
             const float S4 = (q[2][4] + q[2][0]) + (q[4][2] + q[0][2]);
             const float S5 = ((q[3][4] + q[3][0]) + (q[1][4] + q[1][0])) +
                              ((q[4][3] + q[4][1]) + (q[0][3] + q[0][1]));
             const float S8 = (q[4][4] + q[4][0]) + (q[0][4] + q[0][0]);
-            const double pc = pr + (double)q[2][2];
-            const double b1 = K0 * pc + K1 * (4 * pr + (double)S1) + K2 * (4 * pr + (double)S2);
-            const double b2 =
-                K4 * (4 * pr + (double)S4) + K5 * (8 * pr + (double)S5) + K8 * (4 * pr + (double)S8);
-            v[0] += 0.5 * pc * b1;
-            v[1] += 0.5 * pc * b2;
-            v[2] += (double)a.half_A1 * pc * pc;
-            float f[9];
-            load_site_xy(f, g, a.pitch, x, y);
+            Two pc{a.psi_ref, 0.f};
+            two_add(pc, q[2][2], 0.f);
+            Two b1 = k.cs, b2 = k.cm;
+            two_fma(b1, k.K0, pc);
+            two_fma(b1, k.K1, S1);
+            two_fma(b1, k.K2, S2);
+            two_fma(b2, k.K4, S4);
+            two_fma(b2, k.K5, S5);
+            two_fma(b2, k.K8, S8);
+            two_fma(es, pc, b1);
+            two_fma(em, pc, b2);
+            two_fma(eb, pc, pc);
             const float d =
                 ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-            v[3] += (double)d;
+            two_add(ms, d, 0.f);
         }
     }
+    double v[4] = {0.5 * value(es), 0.5 * value(em), (double)a.half_A1 * value(eb), value(ms)};
     if (last_block_total<256>(v, a.partials, a.counter, gridDim.x * gridDim.y)) {
         out4[0] = v[0];
         out4[1] = v[1];
@@ -698,12 +713,21 @@ cudaError_t delta_energy(const T* g, const float* dpsi, int nx, int ny, const St
     StepArgs<T> b = a;
     b.partials = partials;
     b.counter = counter;
-    // at most 152 x 16 CTAs (the state's partial buffer holds at least that many)
+    // one wave of resident CTAs (the state's partial buffer holds twice as many), so that
+    // the FP64 sums above the threads are few
     int bx = (nx + 255) / 256;
     if (bx > 32) bx = 32;
-    int by = 152 * 16 / bx;
+    int by = 152 * 8 / bx;
     if (by > ny) by = ny;
-    k_delta_energy<T><<<dim3(bx, by), 256, 0, s>>>(g, dpsi, b, out4);
+    auto host_two = [](double v) {
+        const float h = (float)v;
+        return Two{h, (float)(v - (double)h)};
+    };
+    const double pr = a.psi_ref, K1 = a.K1, K2 = a.K2, K4 = a.K4, K5 = a.K5, K8 = a.K8;
+    const EnergyArgs k{host_two(a.K0), host_two(K1), host_two(K2), host_two(K4), host_two(K5),
+                       host_two(K8), host_two(pr * (4 * K1 + 4 * K2)),
+                       host_two(pr * (4 * K4 + 8 * K5 + 4 * K8))};
+    k_delta_energy<T><<<dim3(bx, by), 256, 0, s>>>(g, dpsi, b, k, out4);
     return cudaGetLastError();
 }
 
