@@ -211,7 +211,7 @@ lb_status lb_load_state(lb_state* s, const void* src, size_t bytes);
  *   grad_rho      N doubles, host or device: dJ/drho_init(x)
  *   grad_G        host doubles {dJ/dG1, dJ/dG2}
  * Working memory (about 40 N (steps/C + C) bytes) is allocated for the call.
- * Errors: LB_ERR_ARG, LB_ERR_STATE (not FP32, t != 0, poisoned), LB_ERR_OOM,
+ * Errors: LB_ERR_ARG, LB_ERR_STATE (not FP32, t != 0, poisoned), LB_ERR_OOM, LB_ERR_TIMEOUT,
  * LB_ERR_CUDA, LB_ERR_NONFINITE. */
 lb_status lb_adjoint(lb_state* s, long steps, const double* rho_target, int checkpoint_every,
                      double* J, double* grad_rho, double* grad_G);

@@ -292,6 +292,12 @@ lb_status step_fp32(lb_state* s, long n)
     return LB_OK;
 }
 
+}  // namespace
+
+lb_status lbsc::advance_delta(lb_state* s, long n) { return step_fp32(s, n); }
+
+namespace {
+
 Fp64Args make64(const lb_state* s)
 {
     Fp64Args a;

@@ -286,6 +286,56 @@ __device__ __forceinline__ float dpsi_of(float d, const StepArgs<T>& a)
     return a.cpsi * expm1f(-d * a.inv_rho0);
 }
 
+// Halo exchange words. A value travels with the number of the step it belongs to, in one
+// naturally aligned access that is never torn, so a reader needs no barrier or fence: it
+// polls the word until it carries the step's number.
+__device__ __forceinline__ void put_word(uint2* p, float v, unsigned tag)
+{
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p),
+                 "l"((unsigned long long)tag << 32 | __float_as_uint(v))
+                 : "memory");
+}
+__device__ __forceinline__ uint2 get_word(const uint2* p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return make_uint2((unsigned)v, (unsigned)(v >> 32));
+}
+__device__ __forceinline__ void put_word(uint4* p, float a, float b, float c, unsigned tag)
+{
+    asm volatile(
+        "{ .reg .b128 v; mov.b128 v, {%1, %2}; st.relaxed.gpu.global.b128 [%0], v; }" ::"l"(p),
+        "l"((unsigned long long)__float_as_uint(b) << 32 | __float_as_uint(a)),
+        "l"((unsigned long long)tag << 32 | __float_as_uint(c))
+        : "memory");
+}
+__device__ __forceinline__ uint4 get_word(const uint4* p)
+{
+    unsigned long long lo, hi;
+    asm volatile("{ .reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v; }"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+}
+
+// Bounded wait: counts the polls, reads the clock every 256 of them, and once the state's
+// wait limit has passed or another CTA has given up flags the state and the CTA (*fail).
+template <typename T>
+__device__ __forceinline__ bool wait_over(const StepArgs<T>& a, int* fail, unsigned& polls,
+                                          long long& t_end)
+{
+    if ((++polls & 255u) == 0) {
+        const long long now = clock64();
+        if (t_end == 0) t_end = now + a.wait_cycles;
+        if (now > t_end || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
+            atomicOr(a.err, 1);
+            *reinterpret_cast<volatile int*>(fail) = 1;
+        }
+    }
+    return *reinterpret_cast<volatile int*>(fail) != 0;
+}
+
 // Unevaluated sums hi + lo of two FP32 values: products and sums of FP32 terms to about
 // 2^-46 of their magnitude on the FP32 pipe, where FP64 (64 times slower on this part)
 // would bound a kernel that streams memory (TwoSum: Knuth; TwoProduct with a fused

@@ -209,6 +209,10 @@ cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x,
                           cudaStream_t s);
 cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps,
                           cudaStream_t s);
+// The same without trace rows, every state before its step kept in `states`: [steps][4][N],
+// dpsi, density deviation and the momentum negated (x, y).
+cudaError_t fp32_resident_kept(const StepArgs<float>& a, ResidentBuf& b, int steps, float* states,
+                               cudaStream_t s);
 // bulk-copy pipelined step (lb_bulk.cu)
 bool bulk_supported(int nx, int ny, int elem_bytes, int block_x);
 int bulk_grid_blocks(int nx, int ny, int elem_bytes, Fp32Launch L);
@@ -302,6 +306,8 @@ void* state_alloc(lb_state* s, size_t bytes);
 }  // namespace lbsc
 
 namespace lbsc {
+// Take n steps of an FP32 or FP16 state, several per launch where that pays (lb_step).
+lb_status advance_delta(lb_state* s, long n);
 template <typename T>
 StepArgs<T> state_args(const lb_state* s, int cur);   // arguments of a step from buffers `cur`
 size_t elem_size(lb_precision p);

@@ -36,19 +36,25 @@ __host__ __device__ inline PackedArgs packed_args(const StepArgs<T>& a)
                       d(a.rho_ref), d(a.psi_ref), d(a.omega), d(a.omc), d(a.inv_omega)};
 }
 
-// Force sums of force_energy<false> for the columns x, x + 1. A[k], B[k], C[k]
-// are dpsi of columns (x-2, x-1), (x, x+1), (x+2, x+3) in row y + k - 2: the
-// stencil offsets -2, 0 and +2 are whole pairs; the differences that pair an odd
-// offset are formed one half at a time from the pairs' halves.
-__device__ __forceinline__ void force_sums2(const float2 A[5], const float2 B[5], const float2 C[5],
-                                            const PackedArgs& k, float2& Sx, float2& Sy)
+// The twelve pair differences of the force stencil for the columns x, x + 1. A[k],
+// B[k], C[k] are the field's columns (x-2, x-1), (x, x+1), (x+2, x+3) in row y + k - 2: the
+// stencil offsets -2, 0 and +2 are whole pairs; the differences that pair an odd offset
+// are formed one half at a time from the pairs' halves.
+struct Diffs2 {
+    float2 d10, d01, d20, d02;   // (c) - (-c) for c = (1,0), (0,1), (2,0), (0,2)
+    float2 sum1, dif1;           // (1,1) and (1,-1): sum and difference
+    float2 mx, my;               // |c|^2 = 5: the x and y combinations
+    float2 sum8, dif8;           // (2,2) and (2,-2)
+};
+__device__ __forceinline__ Diffs2 diffs2(const float2 A[5], const float2 B[5], const float2 C[5])
 {
-    const float2 d10 = make_float2(B[2].y - A[2].y, C[2].x - B[2].x);
-    const float2 d01 = sub2(B[3], B[1]);
+    Diffs2 r;
+    r.d10 = make_float2(B[2].y - A[2].y, C[2].x - B[2].x);
+    r.d01 = sub2(B[3], B[1]);
     const float2 d11 = make_float2(B[3].y - A[1].y, C[3].x - B[1].x);
     const float2 d1m = make_float2(B[1].y - A[3].y, C[1].x - B[3].x);
-    const float2 d20 = sub2(C[2], A[2]);
-    const float2 d02 = sub2(B[4], B[0]);
+    r.d20 = sub2(C[2], A[2]);
+    r.d02 = sub2(B[4], B[0]);
     const float2 da = sub2(C[3], A[1]);
     const float2 db = make_float2(B[4].y - A[0].y, C[4].x - B[0].x);
     const float2 dc = make_float2(A[4].y - B[0].y, B[4].x - C[0].x);
@@ -56,14 +62,31 @@ __device__ __forceinline__ void force_sums2(const float2 A[5], const float2 B[5]
     const float2 e1 = sub2(C[4], A[0]);
     const float2 e2 = sub2(C[0], A[4]);
     const float2 two = dup2(2.f);
-    float2 sx = fma2(k.K1, d10, mul2(k.K2, add2(d11, d1m)));
-    float2 sy = fma2(k.K1, d01, mul2(k.K2, sub2(d11, d1m)));
-    sx = fma2(k.K4x2, d20, sx);
-    sy = fma2(k.K4x2, d02, sy);
-    sx = fma2(k.K5, fma2(two, sub2(da, dd), sub2(db, dc)), sx);
-    sy = fma2(k.K5, fma2(two, add2(db, dc), add2(da, dd)), sy);
-    Sx = fma2(k.K8x2, add2(e1, e2), sx);
-    Sy = fma2(k.K8x2, sub2(e1, e2), sy);
+    r.sum1 = add2(d11, d1m);
+    r.dif1 = sub2(d11, d1m);
+    r.mx = fma2(two, sub2(da, dd), sub2(db, dc));
+    r.my = fma2(two, add2(db, dc), add2(da, dd));
+    r.sum8 = add2(e1, e2);
+    r.dif8 = sub2(e1, e2);
+    return r;
+}
+// The x and y force sums of force_sums / force_energy<false> from the differences
+__device__ __forceinline__ float2 sum_x2(const Diffs2& r, const PackedArgs& k)
+{
+    const float2 s = fma2(k.K4x2, r.d20, fma2(k.K1, r.d10, mul2(k.K2, r.sum1)));
+    return fma2(k.K8x2, r.sum8, fma2(k.K5, r.mx, s));
+}
+__device__ __forceinline__ float2 sum_y2(const Diffs2& r, const PackedArgs& k)
+{
+    const float2 s = fma2(k.K4x2, r.d02, fma2(k.K1, r.d01, mul2(k.K2, r.dif1)));
+    return fma2(k.K8x2, r.dif8, fma2(k.K5, r.my, s));
+}
+__device__ __forceinline__ void force_sums2(const float2 A[5], const float2 B[5], const float2 C[5],
+                                            const PackedArgs& k, float2& Sx, float2& Sy)
+{
+    const Diffs2 r = diffs2(A, B, C);
+    Sx = sum_x2(r, k);
+    Sy = sum_y2(r, k);
 }
 
 // -1/x of both halves, 1/x rounded to nearest as __frcp_rn gives it: one Newton

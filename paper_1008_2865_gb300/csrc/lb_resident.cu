@@ -37,39 +37,6 @@ using namespace dev;
 
 constexpr int kResThreads = 768;   // at most
 
-// Halo exchange words. A value travels with the number of the step it belongs to, in one
-// naturally aligned access that is never torn, so a reader needs no barrier or fence: it
-// polls the word until it carries the step's number.
-__device__ __forceinline__ void put_word(uint2* p, float v, unsigned tag)
-{
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p),
-                 "l"((unsigned long long)tag << 32 | __float_as_uint(v))
-                 : "memory");
-}
-__device__ __forceinline__ uint2 get_word(const uint2* p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return make_uint2((unsigned)v, (unsigned)(v >> 32));
-}
-__device__ __forceinline__ void put_word(uint4* p, float a, float b, float c, unsigned tag)
-{
-    asm volatile(
-        "{ .reg .b128 v; mov.b128 v, {%1, %2}; st.relaxed.gpu.global.b128 [%0], v; }" ::"l"(p),
-        "l"((unsigned long long)__float_as_uint(b) << 32 | __float_as_uint(a)),
-        "l"((unsigned long long)tag << 32 | __float_as_uint(c))
-        : "memory");
-}
-__device__ __forceinline__ uint4 get_word(const uint4* p)
-{
-    unsigned long long lo, hi;
-    asm volatile("{ .reg .b128 v; ld.relaxed.gpu.global.b128 v, [%2]; mov.b128 {%0, %1}, v; }"
-                 : "=l"(lo), "=l"(hi)
-                 : "l"(p)
-                 : "memory");
-    return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
-}
-
 template <typename T>
 struct ResArgs {
     StepArgs<T> a;
@@ -79,8 +46,9 @@ struct ResArgs {
     unsigned tag;          // steps exchanged before this launch
     uint2* llp;            // [2][N] dpsi halo words
     uint4* llm;            // [2][NQ][N] moments (omega = 1) or populations halo words
-    float* dump;           // [rows][2][N] dpsi and density deviation of the states with a trace row
-    int trace_every;
+    float* dump;           // [rows][planes][N] of the states kept: dpsi, density deviation, and
+    int planes;            // with four planes the momentum, negated
+    int keep_every;        // states t with t % keep_every == 0 are kept; 0: none
 };
 
 template <bool OM1>
@@ -225,14 +193,22 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const ResArgs<T> A)
                 mo = moments2(f);
             }
             if (traced && j >= 1 && j <= h) {
-                float* d0 = A.dump + (size_t)row * 2 * N + (size_t)(y0 + j - 1) * nx + x0 + i - 2;
+                float* d0 = A.dump + (size_t)row * A.planes * N + (size_t)(y0 + j - 1) * nx + x0 + i - 2;
                 if (i >= 2 && i < w + 2) {
                     d0[0] = Bk[2].x;
                     d0[N] = mo.d.x;
+                    if (A.planes == 4) {
+                        d0[2 * (size_t)N] = mo.jx.x;
+                        d0[3 * (size_t)N] = mo.jy.x;
+                    }
                 }
                 if (i + 1 >= 2 && i + 1 < w + 2) {
                     d0[1] = Bk[2].y;
                     d0[N + 1] = mo.d.y;
+                    if (A.planes == 4) {
+                        d0[2 * (size_t)N + 1] = mo.jx.y;
+                        d0[3 * (size_t)N + 1] = mo.jy.y;
+                    }
                 }
             }
             float2 gs[9];
@@ -242,7 +218,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const ResArgs<T> A)
             for (int v = 0; v < 9; ++v) put2(g + v * S, gs[v]);
         }
     };
-    auto is_traced = [&](int s) { return A.trace_every > 0 && (a.t + s) % A.trace_every == 0; };
+    auto is_traced = [&](int s) { return A.keep_every > 0 && (a.t + s) % A.keep_every == 0; };
     bool traced = is_traced(0);
     collide(0, en, traced);
     row += traced;
@@ -338,17 +314,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const ResArgs<T> A)
         collide(0, nfree, traced);
         long long t_end = 0;
         unsigned polls = 0;
-        auto give_up = [&]() -> bool {   // bounded wait: the clock is read every 256 polls
-            if ((++polls & 255u) == 0) {
-                const long long now = clock64();
-                if (t_end == 0) t_end = now + a.wait_cycles;
-                if (now > t_end || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
-                    atomicOr(a.err, 1);
-                    s_fail = 1;
-                }
-            }
-            return *reinterpret_cast<volatile int*>(&s_fail) != 0;
-        };
+        auto give_up = [&]() { return wait_over(a, &s_fail, polls, t_end); };
         for (int q = tid; q < nm * kQuads<OM1> + np; q += nt) {
             if (q < nm * kQuads<OM1>) {
                 const int u = OM1 ? 0 : q / nm;
@@ -507,8 +473,11 @@ cudaError_t launch_resident(const ResArgs<T>& A, int grid, int threads, size_t s
     return cudaLaunchKernelEx(&cfg, k_resident<T, OM1>, A);
 }
 
+// `steps` steps from a's buffers; states with a trace row, or all of them as four planes
+// each, are left in `dump`.
 template <typename T>
-cudaError_t resident_steps(const StepArgs<T>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
+cudaError_t resident_launch(const StepArgs<T>& a, ResidentBuf& b, int steps, float* dump, int planes,
+                            int keep_every, cudaStream_t s)
 {
     ResArgs<T> A{};
     A.a = a;
@@ -520,8 +489,9 @@ cudaError_t resident_steps(const StepArgs<T>& a, ResidentBuf& b, int block_x, in
     A.tag = b.tag;
     A.llp = b.llp;
     A.llm = b.llm;
-    A.dump = b.dump;
-    A.trace_every = b.trace_every;
+    A.dump = dump;
+    A.planes = planes;
+    A.keep_every = keep_every;
     b.tag += (unsigned)steps;
     const bool om1 = a.omega == 1.0f;
     const size_t smem = res_smem(b.tw, b.th, om1);
@@ -532,8 +502,14 @@ cudaError_t resident_steps(const StepArgs<T>& a, ResidentBuf& b, int block_x, in
     const int words = halo_psi(b.tw, b.th) + (om1 ? 1 : 3) * halo_mom(b.tw, b.th);
     int threads = ((pairs > words ? pairs : words) + 31) / 32 * 32;
     threads = threads < 256 ? 256 : threads > kResThreads ? kResThreads : threads;
-    const cudaError_t e = om1 ? launch_resident<T, true>(A, b.gx * b.gy, threads, smem, s)
-                              : launch_resident<T, false>(A, b.gx * b.gy, threads, smem, s);
+    return om1 ? launch_resident<T, true>(A, b.gx * b.gy, threads, smem, s)
+               : launch_resident<T, false>(A, b.gx * b.gy, threads, smem, s);
+}
+
+template <typename T>
+cudaError_t resident_steps(const StepArgs<T>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
+{
+    const cudaError_t e = resident_launch<T>(a, b, steps, b.dump, 2, b.trace_every, s);
     if (e != cudaSuccess || b.trace_every == 0) return e;
     const long long te = b.trace_every, first = (a.t + te - 1) / te * te;
     const int rows = first < a.t + steps ? (int)((a.t + steps - 1 - first) / te + 1) : 0;
@@ -580,6 +556,11 @@ size_t resident_words(long long n, bool om1) { return (size_t)n * 2 * (sizeof(ui
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
 {
     return resident_steps<float>(a, b, block_x, steps, s);
+}
+cudaError_t fp32_resident_kept(const StepArgs<float>& a, ResidentBuf& b, int steps, float* states,
+                               cudaStream_t s)
+{
+    return resident_launch<float>(a, b, steps, states, 4, 1, s);
 }
 cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
 {
