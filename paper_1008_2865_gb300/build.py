@@ -25,6 +25,7 @@ UNITS = {
     "lb_fp32.cu": [],
     "lb_pair.cu": [],
     "lb_resident.cu": [],
+    "lb_trace.cu": [],
     "lb_bulk.cu": [],
     "lb_batch.cu": [],
     "lb_adjoint.cu": [],

@@ -178,6 +178,7 @@ StepArgs<T> state_args(const lb_state* s, int cur)
     a.err = s->err;
     a.wait_cycles = s->wait_cycles;
     a.skip_unit0 = s->skip_unit0;
+    a.dev = s->dev;
     return a;
 }
 
@@ -256,6 +257,19 @@ lb_status step_resident(lb_state* s, long n)
     return LB_OK;
 }
 
+// Steps t and t + 1, and the trace row of state t if it has one.
+template <typename T>
+cudaError_t pair_step(lb_state* s, bool traced)
+{
+    const StepArgs<T> a = make_args<T>(s);
+    cudaError_t e;
+    if constexpr (sizeof(T) == 4) e = fp32_step_pair(a, traced, s->stream);
+    else e = fp16_step_pair(a, traced, s->stream);
+    if (e != cudaSuccess || !traced) return e;
+    const TraceRows r{a.dpsi_in, a.dev, 0, 1, s->t, 1, s->launch.block_x, s->partials, s->counter};
+    return trace_rows<T>(a, r, s->stream);
+}
+
 lb_status step_fp32(lb_state* s, long n)
 {
     // in a stream capture every step is a launch of its own, so that a graph of an even
@@ -266,13 +280,12 @@ lb_status step_fp32(lb_state* s, long n)
         const bool reduce = s->p.trace_every > 0 && (s->t % s->p.trace_every) == 0;
         cudaError_t e;
         const bool bulk = s->launch.pipeline == 1;
-        // two steps without a trace row of their own go through the lattice together
-        // (lb_pair.cu): the same fields bit for bit, half the memory traffic
+        // two steps go through the lattice together (lb_pair.cu) unless the second state
+        // has a trace row: the same fields bit for bit, half the memory traffic
         const bool next_reduces =
             s->p.trace_every > 0 && ((s->t + 1) % s->p.trace_every) == 0;
-        if (many && !reduce && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
-            e = s->p.prec == LB_FP32 ? fp32_step_pair(make_args<float>(s), s->stream)
-                                     : fp16_step_pair(make_args<__half>(s), s->stream);
+        if (many && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
+            e = s->p.prec == LB_FP32 ? pair_step<float>(s, reduce) : pair_step<__half>(s, reduce);
             if (e != cudaSuccess) return fail_cuda(s);
             s->cur ^= 1;
             s->t += 2;
@@ -386,7 +399,7 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     s->max_cta_rows = (p->ny + kMinRows - 1) / kMinRows;
     s->partials_cap += (size_t)s->max_cta_rows;
     bool ok = alloc((void**)&s->partials, 4 * sizeof(double) * s->partials_cap) &&
-              alloc((void**)&s->counter, sizeof(unsigned int)) &&
+              alloc((void**)&s->counter, 2 * sizeof(unsigned int)) &&
               alloc((void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols) &&
               alloc((void**)&s->trace_count, sizeof(int)) &&
               alloc((void**)&s->res, 4 * sizeof(double)) && alloc((void**)&s->flag, sizeof(int)) &&
@@ -399,9 +412,11 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     } else if (ok) {
         const size_t es = elem_size(p->prec);
         const size_t gb = es * (size_t)g_elems(p->nx, p->ny);
+        const size_t dev_at = ((size_t)N + 63) / 64 * 64;   // aligned as a buffer of its own
         ok = alloc(&s->g[0], gb) && alloc(&s->g[1], gb) &&
              alloc((void**)&s->dpsi[0], sizeof(float) * N) &&
-             alloc((void**)&s->dpsi[1], sizeof(float) * N);
+             alloc((void**)&s->dpsi[1], sizeof(float) * (p->trace_every > 0 ? dev_at + N : N));
+        if (p->trace_every > 0) s->dev = s->dpsi[1] + dev_at;
     }
     ResidentBuf& rb = s->res_buf;
     size_t word_bytes = 0;
@@ -452,7 +467,7 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     };
     if (cudaMemcpyAsync(rho_in, rho_init, sizeof(double) * N, cudaMemcpyDefault, s->stream) !=
             cudaSuccess ||
-        cudaMemsetAsync(s->counter, 0, sizeof(unsigned int), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->counter, 0, 2 * sizeof(unsigned int), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->trace_count, 0, sizeof(int), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess ||

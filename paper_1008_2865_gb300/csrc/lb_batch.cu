@@ -153,8 +153,23 @@ BatchLaunch<T> batch_launch(const lb_batch* b, int cur)
                           b->num_sms, b->alternate};
 }
 
+// Steps t and t + 1 of every replica; the trace row of state t, if it has one, follows.
+template <typename T>
+cudaError_t enqueue_pair(const lb_batch* b, cudaStream_t s, int cur, bool traced)
+{
+    const BatchLaunch<T> L = batch_launch<T>(b, cur);
+    cudaError_t e;
+    if constexpr (sizeof(T) == 4)
+        e = fp32_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, traced, s);
+    else
+        e = fp16_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, traced, s);
+    if (e == cudaSuccess && traced) e = batch_trace_partials<T>(L, s);
+    if (e == cudaSuccess && traced) e = batch_reduce<T>(L, s);
+    return e;
+}
+
 // Enqueue step t (buffers `cur` in) of every replica on stream s, or (`pairs`) steps t and
-// t + 1 together when `left` allows and neither appends a trace row; returns through `taken`
+// t + 1 together when `left` allows and state t + 1 has no trace row; returns through `taken`
 // how many steps that was. Either way the buffers swap once.
 cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cur, long long left,
                           bool pairs, int& taken)
@@ -162,15 +177,12 @@ cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cu
     const int te = b->trace_every;
     const bool reduce = te > 0 && t % te == 0;
     const bool next_reduces = te > 0 && (t + 1) % te == 0;
-    taken = pairs && !reduce && !next_reduces && left >= 2 ? 2 : 1;
-    if (b->prec == LB_FP32) {
-        const BatchLaunch<float> L = batch_launch<float>(b, cur);
-        return taken == 2 ? fp32_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, s)
-                          : fp32_batch_step(L, reduce, s);
-    }
-    const BatchLaunch<__half> L = batch_launch<__half>(b, cur);
-    return taken == 2 ? fp16_batch_pair(L, b->d_pair_tiles, b->npair_tiles, b->odd, s)
-                      : fp16_batch_step(L, reduce, s);
+    taken = pairs && !next_reduces && left >= 2 ? 2 : 1;
+    if (taken == 2)
+        return b->prec == LB_FP32 ? enqueue_pair<float>(b, s, cur, reduce)
+                                  : enqueue_pair<__half>(b, s, cur, reduce);
+    return b->prec == LB_FP32 ? fp32_batch_step(batch_launch<float>(b, cur), reduce, s)
+                              : fp16_batch_step(batch_launch<__half>(b, cur), reduce, s);
 }
 
 // Capture one period of steps starting at an aligned time (t % period == 0) with

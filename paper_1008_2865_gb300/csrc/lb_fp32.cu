@@ -615,6 +615,25 @@ cudaError_t fp16_step(const StepArgs<__half>& a, Fp32Launch L, bool reduce, cuda
     return launch_step<__half>(a, L, reduce, s);
 }
 
+template <typename T>
+cudaError_t batch_reduce(const BatchLaunch<T>& b, cudaStream_t s)
+{
+    auto go = [&](auto kern, int bx) {
+        kern<<<b.nrows, bx, 0, s>>>(b.tile_partials, b.reps, b.rowmap, b.trace_every);
+        return cudaGetLastError();
+    };
+    switch (b.block_x) {
+    case 64: return go(k_batch_reduce<64>, 64);
+    case 96: return go(k_batch_reduce<96>, 96);
+    case 128: return go(k_batch_reduce<128>, 128);
+    case 192: return go(k_batch_reduce<192>, 192);
+    case 256: return go(k_batch_reduce<256>, 256);
+    default: return cudaErrorInvalidValue;
+    }
+}
+template cudaError_t batch_reduce<float>(const BatchLaunch<float>&, cudaStream_t);
+template cudaError_t batch_reduce<__half>(const BatchLaunch<__half>&, cudaStream_t);
+
 template <typename T, int BX>
 cudaError_t launch_batch_bx(const BatchLaunch<T>& b, bool reduce, cudaStream_t s)
 {
@@ -644,9 +663,7 @@ cudaError_t launch_batch_bx(const BatchLaunch<T>& b, bool reduce, cudaStream_t s
             e = b.om1 ? pick(k_step_batch<T, BX, false, true, false>)
                       : pick(k_step_batch<T, BX, false, false, false>);
     }
-    if (e != cudaSuccess || !reduce) return e;
-    k_batch_reduce<BX><<<b.nrows, BX, 0, s>>>(b.tile_partials, b.reps, b.rowmap, b.trace_every);
-    return cudaGetLastError();
+    return e != cudaSuccess || !reduce ? e : batch_reduce<T>(b, s);
 }
 
 template <typename T>

@@ -120,6 +120,7 @@ struct StepArgs {
     int* err;                        // error flags: 1 a wait ran out, 2 a reduction was not finite
     long long wait_cycles;           // clock limit of one wait
     int skip_unit0;                  // test hook: the first row unit's barrier is armed, no copy issued
+    float* __restrict__ dev;         // [ny][nx] density deviations of a traced state (pairs of steps)
 };
 
 // Output rows per CTA accepted by lb_set_launch / lb_batch_set_launch.
@@ -178,8 +179,9 @@ cudaError_t fp16_batch_step(const BatchLaunch<__half>& b, bool reduce, cudaStrea
 // launches of k_step (us per step, single and paired: 250x187 10.1 and 10.2, 512^2 10.3
 // and 9.3, 700^2 12.3 and 10.2).
 inline bool pairs_pay(long long n) { return n >= (1LL << 18); }
-cudaError_t fp32_step_pair(const StepArgs<float>& a, cudaStream_t s);
-cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s);
+// (traced: the density deviations of state t are left in a.dev)
+cudaError_t fp32_step_pair(const StepArgs<float>& a, bool traced, cudaStream_t s);
+cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t s);
 // The same for a batch of any size (its single-step tiles are 32 rows high unless the
 // caller chose otherwise, so even small batches gain: 27 replicas of up to 69^2, 30.7 ->
 // 9.5 us per step; nine 512^2 57.4 -> 28.7; the 96-replica sweep 338 -> 205): `tiles` (pair_tiles: replica, first column, first row, end row)
@@ -187,9 +189,28 @@ cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s);
 void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, bool om1, int num_sms,
                 std::vector<int4>& tiles);
 cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int ntiles, bool odd,
-                            cudaStream_t s);
+                            bool traced, cudaStream_t s);
 cudaError_t fp16_batch_pair(const BatchLaunch<__half>& b, const int4* tiles, int ntiles, bool odd,
-                            cudaStream_t s);
+                            bool traced, cudaStream_t s);
+// Trace rows of kept states (lb_trace.cu), as reduction steps of launch width block_x and
+// a.rows write them: `count` states `apart` values from one another, at t, t + every, ...
+struct TraceRows {
+    const float *dpsi, *dev;
+    size_t apart;
+    int count;
+    long long t;
+    int every;
+    int block_x;
+    double* partials;                     // [count][CTA partials, row totals][4]
+    unsigned int* counters;               // [1 + count], zero between uses
+};
+template <typename T>
+cudaError_t trace_rows(const StepArgs<T>& a, const TraceRows& r, cudaStream_t s);
+// the tile partials of a batch's traced states (from dpsi_in and dev), and their sums
+template <typename T>
+cudaError_t batch_trace_partials(const BatchLaunch<T>& b, cudaStream_t s);
+template <typename T>
+cudaError_t batch_reduce(const BatchLaunch<T>& b, cudaStream_t s);
 // Many steps of a small lattice in one launch (lb_resident.cu): the tiles its CTAs hold
 // and the buffers they exchange through.
 struct ResidentBuf {
@@ -265,6 +286,7 @@ struct lb_state {
     // FP32 / FP16 deviation storage (g tiled, lbsc::g_elems elements each)
     void* g[2] = {nullptr, nullptr};
     float* dpsi[2] = {nullptr, nullptr};
+    float* dev = nullptr;          // density deviations of a traced state (in dpsi[1]'s buffer)
     int cur = 0;
     double rho_ref = 0.0;
     lbsc::Fp32Launch launch{128, 64, 0};

@@ -27,7 +27,10 @@
 // population rows 619 (with an earlier form of the rest).
 //
 // Every site's arithmetic is that of k_step, operation by operation, so the fields
-// are bit-identical to two single steps.
+// are bit-identical to two single steps. If state t has a trace row, stage 1 leaves its
+// density deviations in memory (4 bytes per site) and the row is formed from them and
+// dpsi afterwards (lb_trace.cu): 0.28 ms at 8192^2, against 0.73 ms that a reduction step
+// and a plain one cost more than a pair.
 #include "lb_packed.cuh"
 
 #include <type_traits>
@@ -264,7 +267,7 @@ __device__ __forceinline__ void collide_row(const PackedArgs& k, const float2 (*
     o.l6 = gs[6].y;
 }
 
-template <typename T, int TH, bool OM1, bool ODD>
+template <typename T, int TH, bool OM1, bool ODD, bool TRACE>
 __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs& k, PairShared<T, TH, OM1>& sh, int x0, int y0,
                                           int y1)
 {
@@ -304,6 +307,8 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
     Own o1, o2;
     float2 f1[9];
     f.unpack(f1);
+    // TRACE: the density deviations of state t at the tile's own sites
+    float* dev = TRACE ? a.dev + (long long)(rs + 1) * nx + xa : nullptr;   // row r + 1
     collide_row<OM1, T, TH>(k, sh.win[0], rs, moments2(f1), f1, sh.exR[0][rs & 1], sh.exL[0][rs & 1], o1);
     load_cols<ODD>(f, a.g_in + la, c);
     la = la + P == NP ? 0 : la + P;
@@ -350,6 +355,17 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
         if (S1) {
             f.unpack(f1);
             m1 = moments2(f1);
+            if (TRACE) {
+                if (outa && r + 1 >= y0 && r + 1 < y1) {
+                    if (!ODD) {
+                        *reinterpret_cast<float2*>(dev) = m1.d;
+                    } else {
+                        dev[0] = m1.d.x;
+                        if (outb) dev[1] = m1.d.y;
+                    }
+                }
+                dev += nx;
+            }
         }
         if (S1 && r + 2 <= y1 + 3) load_cols<ODD>(f, a.g_in + la, c);
         la = la + P == NP ? 0 : la + P;
@@ -503,13 +519,13 @@ template <typename T, bool OM1>
 constexpr int kPairThreads = OM1 && sizeof(T) == 2 ? 512 : 384;
 constexpr int kTH = 64;   // threads per CTA
 
-template <typename T, int TH, bool OM1, bool ODD>
+template <typename T, int TH, bool OM1, bool ODD, bool TRACE>
 __global__ void __launch_bounds__(TH, kPairThreads<T, OM1> / TH)
     k_step2(const StepArgs<T> a, const PackedArgs k, int rows)
 {
     __shared__ PairShared<T, TH, OM1> sh;
     const int y0 = blockIdx.y * rows;
-    pair_tile<T, TH, OM1, ODD>(a, k, sh, blockIdx.x * (2 * TH - 8), y0, min(y0 + rows, a.ny));
+    pair_tile<T, TH, OM1, ODD, TRACE>(a, k, sh, blockIdx.x * (2 * TH - 8), y0, min(y0 + rows, a.ny));
 }
 
 // Output rows per CTA: one wave of resident CTAs, because a chunk's ends cost ten rows
@@ -532,25 +548,38 @@ int pair_rows(int nx, int ny, bool om1)
     return rows < 8 ? 8 : rows;
 }
 
+// f(omega == 1, odd nx, traced) with the three as compile-time constants
+template <typename F>
+cudaError_t with_flags(bool om1, bool odd, bool traced, F f)
+{
+    using Y = std::true_type;
+    using N = std::false_type;
+    if (traced) {
+        if (om1) return odd ? f(Y{}, Y{}, Y{}) : f(Y{}, N{}, Y{});
+        return odd ? f(N{}, Y{}, Y{}) : f(N{}, N{}, Y{});
+    }
+    if (om1) return odd ? f(Y{}, Y{}, N{}) : f(Y{}, N{}, N{});
+    return odd ? f(N{}, Y{}, N{}) : f(N{}, N{}, N{});
+}
+
 template <typename T>
-cudaError_t launch_pair(const StepArgs<T>& a, cudaStream_t s)
+cudaError_t launch_pair(const StepArgs<T>& a, bool traced, cudaStream_t s)
 {
     constexpr int W = 2 * kTH - 8;
-    const bool om1 = a.omega == 1.0f, odd = a.nx & 1;
+    const bool om1 = a.omega == 1.0f;
     const int rows = pair_rows<T>(a.nx, a.ny, om1);
     const dim3 grid((a.nx + W - 1) / W, (a.ny + rows - 1) / rows);
-    const PackedArgs k = packed_args(a);
-    if (om1 && odd) k_step2<T, kTH, true, true><<<grid, kTH, 0, s>>>(a, k, rows);
-    else if (om1) k_step2<T, kTH, true, false><<<grid, kTH, 0, s>>>(a, k, rows);
-    else if (odd) k_step2<T, kTH, false, true><<<grid, kTH, 0, s>>>(a, k, rows);
-    else k_step2<T, kTH, false, false><<<grid, kTH, 0, s>>>(a, k, rows);
-    return cudaGetLastError();
+    return with_flags(om1, a.nx & 1, traced, [&](auto o, auto d, auto t) {
+        k_step2<T, kTH, decltype(o)::value, decltype(d)::value, decltype(t)::value>
+            <<<grid, kTH, 0, s>>>(a, packed_args(a), rows);
+        return cudaGetLastError();
+    });
 }
 
 // The pairs of a batch: a persistent grid strides over a work list of tiles (replica,
 // first column, first row, end row) of every replica. The replica's arguments are
 // staged in shared memory by warp 0 when the replica changes.
-template <typename T, bool OM1, bool ODD>
+template <typename T, bool OM1, bool ODD, bool TRACE>
 __global__ void __launch_bounds__(kTH, kPairThreads<T, OM1> / kTH)
     k_step2_batch(const StepArgs<T>* __restrict__ args, const int4* __restrict__ tiles, int ntiles)
 {
@@ -575,21 +604,21 @@ __global__ void __launch_bounds__(kTH, kPairThreads<T, OM1> / kTH)
         }
         __syncthreads();
         const StepArgs<T> a = sa;
-        pair_tile<T, kTH, OM1, ODD>(a, sk, sh, tl.y, tl.z, tl.w);
+        pair_tile<T, kTH, OM1, ODD, TRACE>(a, sk, sh, tl.y, tl.z, tl.w);
     }
 }
 
 template <typename T>
 cudaError_t launch_batch_pair(const BatchLaunch<T>& b, const int4* tiles, int ntiles, bool odd,
-                              cudaStream_t s)
+                              bool traced, cudaStream_t s)
 {
     const int per_sm = (b.om1 ? kPairThreads<T, true> : kPairThreads<T, false>) / kTH;
     const int grid = ntiles < per_sm * b.num_sms ? ntiles : per_sm * b.num_sms;
-    if (b.om1 && odd) k_step2_batch<T, true, true><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
-    else if (b.om1) k_step2_batch<T, true, false><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
-    else if (odd) k_step2_batch<T, false, true><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
-    else k_step2_batch<T, false, false><<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
-    return cudaGetLastError();
+    return with_flags(b.om1, odd, traced, [&](auto o, auto d, auto t) {
+        k_step2_batch<T, decltype(o)::value, decltype(d)::value, decltype(t)::value>
+            <<<grid, kTH, 0, s>>>(b.args, tiles, ntiles);
+        return cudaGetLastError();
+    });
 }
 
 }  // namespace
@@ -633,17 +662,23 @@ void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, b
 }
 
 cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int ntiles, bool odd,
-                            cudaStream_t s)
+                            bool traced, cudaStream_t s)
 {
-    return launch_batch_pair<float>(b, tiles, ntiles, odd, s);
+    return launch_batch_pair<float>(b, tiles, ntiles, odd, traced, s);
 }
 cudaError_t fp16_batch_pair(const BatchLaunch<__half>& b, const int4* tiles, int ntiles, bool odd,
-                            cudaStream_t s)
+                            bool traced, cudaStream_t s)
 {
-    return launch_batch_pair<__half>(b, tiles, ntiles, odd, s);
+    return launch_batch_pair<__half>(b, tiles, ntiles, odd, traced, s);
 }
 
-cudaError_t fp32_step_pair(const StepArgs<float>& a, cudaStream_t s) { return launch_pair<float>(a, s); }
-cudaError_t fp16_step_pair(const StepArgs<__half>& a, cudaStream_t s) { return launch_pair<__half>(a, s); }
+cudaError_t fp32_step_pair(const StepArgs<float>& a, bool traced, cudaStream_t s)
+{
+    return launch_pair<float>(a, traced, s);
+}
+cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t s)
+{
+    return launch_pair<__half>(a, traced, s);
+}
 
 }  // namespace lbsc

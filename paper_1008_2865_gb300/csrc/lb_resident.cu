@@ -26,8 +26,9 @@
 //
 // Every site's arithmetic is that of k_step, operation by operation, so the fields are
 // bit-identical to single steps. States with a trace row leave their dpsi and density
-// deviation in a buffer; k_trace_partial forms the energies from them afterwards, for
-// all rows of the launch at once, in the order of k_step's threads.
+// deviation in a buffer; trace_rows (lb_trace.cu) forms the
+// energies from them afterwards, for all rows of the launch at once, in the order of
+// k_step's threads.
 #include "lb_packed.cuh"
 
 namespace lbsc {
@@ -340,120 +341,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(const ResArgs<T> A)
     }
 }
 
-// The trace rows of dumped states: CTA (bx, by, row) is CTA (bx, by) of k_step's grid
-// and forms its partial from the dumped dpsi and deviations, thread by thread in the
-// order of k_step's march, so the row is the one the reduction step itself writes.
-template <typename T, int BX>
-__global__ void __launch_bounds__(BX)
-    k_trace_partial(const StepArgs<T> a, const float* __restrict__ dump, double* __restrict__ partials,
-                    int stride, bool alternate)
-{
-    __shared__ double red[4 * BX];
-    const int tid = threadIdx.x, nx = a.nx, ny = a.ny;
-    const float* dpsi = dump + (size_t)blockIdx.z * 2 * a.N;
-    const float* dev = dpsi + a.N;
-    const int x0 = blockIdx.x * (BX - 2), y0 = blockIdx.y * a.rows;
-    const int nrows = min(a.rows, ny - y0);
-    const int x = x0 - 1 + tid;
-    const bool on = tid >= 1 && tid <= min(BX - 2, nx - x0);
-    const bool up = alternate && (blockIdx.y & 1);
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    float es = 0.f, em = 0.f, eb = 0.f, ms = 0.f;
-    if (on) {
-        int xc[5];
-#pragma unroll
-        for (int m = 0; m < 5; ++m) xc[m] = wrapi(x + m - 2, nx);
-        for (int k = 1; k <= nrows; ++k) {
-            const int y = up ? y0 + nrows - k : y0 + k - 1;
-            float q[5][5];
-#pragma unroll
-            for (int r = 0; r < 5; ++r) {
-                const float* src = dpsi + (size_t)wrapi(y + r - 2, ny) * nx;
-#pragma unroll
-                for (int m = 0; m < 5; ++m) q[r][m] = __ldg(src + xc[m]);
-            }
-            const float* rows[5] = {&q[0][2], &q[1][2], &q[2][2], &q[3][2], &q[4][2]};
-            float Sx, Sy;
-            force_energy<true>(rows, a, Sx, Sy, 1.f, a.psi_ref + q[2][2], es, em, eb);
-            ms = fmaf(1.f, __ldg(dev + (size_t)y * nx + x), ms);
-            if ((k & 63) == 63) {
-                v[0] += es;
-                v[1] += em;
-                v[2] += eb;
-                v[3] += ms;
-                es = em = eb = ms = 0.f;
-            }
-        }
-    }
-    v[0] += es;
-    v[1] += em;
-    v[2] += eb;
-    v[3] += ms;
-    block_sum4<BX>(v, red);
-    if (tid == 0) {
-        double* p = partials + 4 * ((size_t)blockIdx.z * stride + (size_t)blockIdx.y * gridDim.x + blockIdx.x);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) p[q] = v[q];
-    }
-}
-
-// The grid sums of dumped states: k_step_total for every trace row (blockIdx.y) at once.
-template <int NT>
-__global__ void __launch_bounds__(NT)
-    k_trace_total(const double* __restrict__ cta, double* __restrict__ rows, int stride, int nbx,
-                  unsigned int* counters, double* trace, int* trace_count, int* err, long long t,
-                  int trace_every, double mass_ref)
-{
-    __shared__ double red[4 * NT];
-    const int nby = gridDim.x, z = blockIdx.y, nz = gridDim.y;
-    double w[4];
-    if (row_then_total<NT>(cta + 4 * (size_t)z * stride, nbx, nby, blockIdx.x,
-                           rows + 4 * (size_t)z * stride, counters + 1 + z, w, red)) {
-        const int c = *reinterpret_cast<volatile int*>(trace_count);
-        const double mass = mass_ref + w[3];
-        double* r = trace + (size_t)((c + z) % kTraceCap) * kTraceCols;
-        r[0] = (double)(t + (long long)z * trace_every);
-        r[1] = mass;
-        r[2] = w[0];
-        r[3] = w[1];
-        r[4] = w[2];
-        if (!isfinite(mass) || !isfinite(w[0]) || !isfinite(w[1])) atomicOr(err, 2);
-        __threadfence();
-        // the last row to finish counts all of them
-        if (atomicAdd(counters, 1u) == (unsigned)nz - 1) {
-            *trace_count = c + nz;
-            *counters = 0u;
-        }
-    }
-}
-
-template <typename T, int BX>
-cudaError_t trace_rows_bx(const StepArgs<T>& a, const ResidentBuf& b, int rows, cudaStream_t s)
-{
-    const dim3 grid((a.nx + BX - 3) / (BX - 2), (a.ny + a.rows - 1) / a.rows, rows);
-    const int stride = (int)(grid.x * grid.y + grid.y);
-    k_trace_partial<T, BX><<<grid, BX, 0, s>>>(a, b.dump, b.partials, stride, marches_alternate(a.N));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_trace_total<BX><<<dim3(grid.y, rows), BX, 0, s>>>(
-        b.partials, b.partials + 4 * (size_t)grid.x * grid.y, stride, (int)grid.x, b.counters, a.trace,
-        a.trace_count, a.err, a.t, b.trace_every, (double)a.N * (double)a.rho_ref);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t trace_rows(const StepArgs<T>& a, const ResidentBuf& b, int block_x, int rows, cudaStream_t s)
-{
-    switch (block_x) {
-    case 64: return trace_rows_bx<T, 64>(a, b, rows, s);
-    case 96: return trace_rows_bx<T, 96>(a, b, rows, s);
-    case 128: return trace_rows_bx<T, 128>(a, b, rows, s);
-    case 192: return trace_rows_bx<T, 192>(a, b, rows, s);
-    case 256: return trace_rows_bx<T, 256>(a, b, rows, s);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
 template <typename T, bool OM1>
 cudaError_t launch_resident(const ResArgs<T>& A, int grid, int threads, size_t smem, cudaStream_t s)
 {
@@ -514,9 +401,17 @@ cudaError_t resident_steps(const StepArgs<T>& a, ResidentBuf& b, int block_x, in
     const long long te = b.trace_every, first = (a.t + te - 1) / te * te;
     const int rows = first < a.t + steps ? (int)((a.t + steps - 1 - first) / te + 1) : 0;
     if (rows == 0) return cudaSuccess;
-    StepArgs<T> at = a;
-    at.t = first;
-    return trace_rows(at, b, block_x, rows, s);
+    TraceRows r{};
+    r.dpsi = b.dump;
+    r.dev = b.dump + a.N;
+    r.apart = 2 * (size_t)a.N;
+    r.count = rows;
+    r.t = first;
+    r.every = b.trace_every;
+    r.block_x = block_x;
+    r.partials = b.partials;
+    r.counters = b.counters;
+    return trace_rows(a, r, s);
 }
 
 }  // namespace
