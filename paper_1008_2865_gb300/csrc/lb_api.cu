@@ -198,22 +198,25 @@ lb_status fail_cuda(lb_state* s)
     return LB_ERR_CUDA;
 }
 
-// Read the kernels' error flags (synchronises the stream): bit 1, a bounded
-// wait ran out (the state is poisoned); bit 2, a fused reduction produced a
-// non-finite mass or energy (the lattice has blown up).
-lb_status check_err(lb_state* s)
+// Read the state's control words (synchronises the stream) and the kernels' error flags
+// among them: bit 1, a bounded wait ran out (the state is poisoned); bit 2, a fused
+// reduction produced a non-finite mass or energy (the lattice has blown up).
+lb_status read_control(lb_state* s, Control& c)
 {
-    int e = 0;
-    if (cudaMemcpyAsync(&e, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream) !=
-            cudaSuccess ||
+    if (cudaMemcpyAsync(&c, s->res, sizeof(c), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         return fail_cuda(s);
-    if (e & 1) {
+    if (c.err & 1) {
         s->poisoned = true;
         return LB_ERR_TIMEOUT;
     }
-    if (e & 2) return LB_ERR_NONFINITE;
-    return LB_OK;
+    return c.err & 2 ? LB_ERR_NONFINITE : LB_OK;
+}
+
+lb_status check_err(lb_state* s)
+{
+    Control c;
+    return read_control(s, c);
 }
 
 #define LB_CUDA(s, call)                          \
@@ -399,11 +402,16 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     s->max_cta_rows = (p->ny + kMinRows - 1) / kMinRows;
     s->partials_cap += (size_t)s->max_cta_rows;
     bool ok = alloc((void**)&s->partials, 4 * sizeof(double) * s->partials_cap) &&
-              alloc((void**)&s->counter, 2 * sizeof(unsigned int)) &&
-              alloc((void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols) &&
-              alloc((void**)&s->trace_count, sizeof(int)) &&
-              alloc((void**)&s->res, 4 * sizeof(double)) && alloc((void**)&s->flag, sizeof(int)) &&
-              alloc((void**)&s->err, sizeof(int));
+              alloc((void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols);
+    Control* ctl = nullptr;
+    ok = ok && alloc((void**)&ctl, sizeof(Control));
+    if (ok) {
+        s->res = ctl->res;
+        s->err = &ctl->err;
+        s->trace_count = &ctl->trace_count;
+        s->flag = &ctl->flag;
+        s->counter = ctl->counter;
+    }
     if (ok && p->prec == LB_FP64) {
         ok = alloc((void**)&s->f64[0], 9 * sizeof(double) * N) &&
              alloc((void**)&s->f64[1], 9 * sizeof(double) * N) &&
@@ -467,26 +475,20 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     };
     if (cudaMemcpyAsync(rho_in, rho_init, sizeof(double) * N, cudaMemcpyDefault, s->stream) !=
             cudaSuccess ||
-        cudaMemsetAsync(s->counter, 0, 2 * sizeof(unsigned int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->trace_count, 0, sizeof(int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(ctl, 0, sizeof(Control), s->stream) != cudaSuccess ||
         (rb.gx > 0 &&
          cudaMemsetAsync(rb.counters, 0, 256 + word_bytes, s->stream) != cudaSuccess))
         return bail(LB_ERR_CUDA);
     if (rho_check_sum(rho_in, N, s->partials, s->counter, s->res, s->flag, s->stream) !=
         cudaSuccess)
         return bail(LB_ERR_CUDA);
-    double sum = 0.0;
-    int flag = 0;
+    Control got{};
     // after this synchronisation the caller's rho_init is no longer read
-    if (cudaMemcpyAsync(&sum, s->res, sizeof(double), cudaMemcpyDeviceToHost, s->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(&flag, s->flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream) !=
-            cudaSuccess ||
+    if (cudaMemcpyAsync(&got, ctl, sizeof(got), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         return bail(LB_ERR_CUDA);
-    if (flag) return bail(LB_ERR_ARG);
+    const double sum = got.res[0];
+    if (got.flag) return bail(LB_ERR_ARG);
     // The reference density is rounded to FP32 once: the kernels add it in FP32,
     // the deviations at init and the mass/field reconstructions use it in FP64,
     // and all of them must mean the same number.
@@ -549,16 +551,12 @@ lb_status lb_energy(lb_state* s, double out[4])
         LB_CUDA(s, delta_energy<__half>(a.g_in, a.dpsi_in, s->p.nx, s->p.ny, a, s->res,
                                         s->partials, s->counter, s->stream));
     }
-    double h[4];
-    LB_CUDA(s, cudaMemcpyAsync(h, s->res, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
-    LB_CUDA(s, cudaStreamSynchronize(s->stream));
-    {
-        const lb_status st = check_err(s);
-        if (st != LB_OK) return st;
-    }
-    for (int k = 0; k < 4; ++k) out[k] = h[k];
+    Control c;
+    const lb_status st = read_control(s, c);
+    if (st != LB_OK) return st;
+    for (int k = 0; k < 4; ++k) out[k] = c.res[k];
     for (int k = 0; k < 4; ++k)
-        if (!std::isfinite(h[k])) return LB_ERR_NONFINITE;
+        if (!std::isfinite(c.res[k])) return LB_ERR_NONFINITE;
     return LB_OK;
 }
 
@@ -582,7 +580,7 @@ lb_status lb_objective(lb_state* s, const double* rho_target, double* J)
                                    cudaMemcpyHostToDevice, s->stream));
         tgt = s->field_tmp;
     }
-    double h[4] = {0.0, 0.0, 0.0, 0.0};
+    double h[2] = {0.0, 0.0};
     if (s->p.prec == LB_FP64) {
         // psi and rho of the current state, the Sec. 5 sums, then the misfit
         const Fp64Args a = make64(s);
@@ -592,23 +590,15 @@ lb_status lb_objective(lb_state* s, const double* rho_target, double* J)
         LB_CUDA(s, cudaMemcpyAsync(h, s->res, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                                    s->stream));
         LB_CUDA(s, misfit64(s->rho64, tgt, N, s->partials, s->counter, s->res, s->stream));
-        LB_CUDA(s, cudaMemcpyAsync(h + 2, s->res, sizeof(double), cudaMemcpyDeviceToHost,
-                                   s->stream));
-        LB_CUDA(s, cudaStreamSynchronize(s->stream));
-        *J = (h[0] + h[1]) + h[2];
     } else {
         // the terminal sums of lb_adjoint (same kernel, grid and order)
         LB_CUDA(s, objective_delta(s, tgt, s->res, s->stream));
-        LB_CUDA(s, cudaMemcpyAsync(h, s->res, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                   s->stream));
-        LB_CUDA(s, cudaStreamSynchronize(s->stream));
-        *J = h[0] + h[1];
     }
-    {
-        const lb_status st = check_err(s);
-        if (st != LB_OK) return st;
-    }
-    return std::isfinite(*J) ? LB_OK : LB_ERR_NONFINITE;
+    Control c;
+    const lb_status st = read_control(s, c);
+    if (st == LB_ERR_CUDA) return st;
+    *J = s->p.prec == LB_FP64 ? (h[0] + h[1]) + c.res[0] : c.res[0] + c.res[1];
+    return st != LB_OK || std::isfinite(*J) ? st : LB_ERR_NONFINITE;
 }
 
 static cudaError_t fields_into(lb_state* s, double* r, double* x, double* y)
@@ -654,7 +644,6 @@ lb_status lb_fields(lb_state* s, double* rho, double* ux, double* uy)
         LB_CUDA(s, cudaMemcpyAsync(outs[k], t, sizeof(double) * N, cudaMemcpyDeviceToHost,
                                    s->stream));
     }
-    LB_CUDA(s, cudaStreamSynchronize(s->stream));
     return check_err(s);
 }
 
@@ -665,10 +654,10 @@ lb_status lb_trace(lb_state* s, double* buf, int cap, int* count)
     if (s->poisoned) return LB_ERR_STATE;
     DeviceScope dev(s->p.device);
     if (!dev.ok) return fail_cuda(s);
-    int total = 0;
-    LB_CUDA(s, cudaMemcpyAsync(&total, s->trace_count, sizeof(int), cudaMemcpyDeviceToHost,
-                               s->stream));
-    LB_CUDA(s, cudaStreamSynchronize(s->stream));
+    Control c;
+    const lb_status st = read_control(s, c);
+    if (st == LB_ERR_CUDA) return st;
+    const int total = c.trace_count;
     const int stored = total < kTraceCap ? total : kTraceCap;
     const int n = stored < cap ? stored : cap;
     // rows total-n .. total-1, oldest first; row r lives in ring slot r % kTraceCap,
@@ -686,7 +675,7 @@ lb_status lb_trace(lb_state* s, double* buf, int cap, int* count)
     }
     LB_CUDA(s, cudaStreamSynchronize(s->stream));
     *count = n;
-    return check_err(s);
+    return st;
 }
 
 namespace {

@@ -275,6 +275,15 @@ cudaError_t fp64_exp_cr(const double* x, double* y, long long n, cudaStream_t s)
 
 }  // namespace lbsc
 
+namespace lbsc {
+// The words of a state the host reads back, together in one transfer, and the counters.
+struct Control {
+    double res[4];
+    int err, trace_count, flag;
+    unsigned int counter[2];
+};
+}  // namespace lbsc
+
 // The state behind the opaque lb_state* of the C ABI (lb_api.cu owns its
 // lifetime; lb_batch.cu drives several of them with one launch per step).
 struct lb_state {
@@ -305,7 +314,7 @@ struct lb_state {
     unsigned int* counter = nullptr;
     double* trace = nullptr;
     int* trace_count = nullptr;
-    double* res = nullptr;         // 4 doubles of results
+    double* res = nullptr;         // 4 doubles of results; err and trace_count follow them
     int* flag = nullptr;
     double* field_tmp = nullptr;   // N doubles, allocated on the first lb_fields into pageable host memory
     // every device buffer of the state, with a guard region on each side
