@@ -321,8 +321,10 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
     T* gp = a.g_out + (long long)(rs - 5) * P;        // g row of stage 2's collision row
 
     // the strip's population tiles of a row, [tl, t1), and past the periodic edge
-    // [0, t2): one thread has them fetched into L2 four rows ahead of their load
-    constexpr int kAhead = 4;
+    // [0, t2): one thread has them fetched into L2 three rows ahead of their load (us per
+    // step at 8192^2 with two, three, four, eight rows: FP16 446, 442, 451, 448; FP32 495,
+    // 497, 501, 536)
+    constexpr int kAhead = 3;
     const int tl = wrapi(x0 - 4, nx) >> 5, tiles = (nx + 31) >> 5;
     const int span = (2 * TH + 31 + 31) / 32;
     const int t1 = min(tl + span, tiles), t2 = min(span - (t1 - tl), tl);
