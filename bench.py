@@ -2,8 +2,8 @@
 
 One "step" is one pass of the whole hot path over the lattice: moments,
 psi, the two-belt force, velocity-shifted BGK collision, streaming (on chip),
-psi of the next state, and (every 10th step) the fused pseudo-energy and mass
-reduction. The workload is the 8192 x 8192 periodic lattice, FP32, G1 = -5,
+psi of the next state, and (every 10th step) the pseudo-energy and mass
+reduction; two steps share a pass over memory. The workload is the 8192 x 8192 periodic lattice, FP32, G1 = -5,
 G2 = 0.6, rho = 0.7 (1 +- 1%) seeded noise — the bandwidth-roofline case.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
@@ -34,7 +34,29 @@ sys.path.insert(0, ROOT)
 NX = NY = 8192
 G1, G2, OMEGA, SEED = -5.0, 0.6, 1.0, 7
 TRACE_EVERY = 10
-BYTES_PER_SITE = 80          # 36 B populations in + 36 B out + 4 B dpsi in + 4 B dpsi out
+# One pass over the lattice (36 B of populations in + 36 B out + 4 B of dpsi in + 4 B out)
+# takes two steps; a state with a trace row adds 4 B written and 8 B read (its density
+# deviations, and both fields for the sums).
+PASS_BYTES = {"fp32": 80, "fp16_delta": 44}
+
+
+def bytes_per_site_step(prec, bulk=False):
+    """Algorithmic bytes per site and step of the benchmark's trace period."""
+    return PASS_BYTES[prec] if bulk else PASS_BYTES[prec] / 2 + 12 / TRACE_EVERY
+
+
+def step_launches(steps):
+    """Kernel launches of lb_step(steps) from an aligned time: pairs of steps, two more
+    kernels for a trace row, single steps where a pair does not fit."""
+    n = t = 0
+    while t < steps:
+        traced, next_traced = t % TRACE_EVERY == 0, (t + 1) % TRACE_EVERY == 0
+        pair = t + 1 < steps and not next_traced
+        n += 1 + (2 if pair else 1) * traced
+        t += 2 if pair else 1
+    return n
+
+
 METRIC = "MLUPS and % HBM roofline (FP32 fused step, 1 GB300); adjoint+batched vs plain"
 WORKLOAD = ("{n}x{n} periodic D2Q9 two-belt Shan-Chen, FP32 (deviation storage), omega=1, "
             "G1=-5.0, G2=0.6, rho=0.7(1+-1%) seeded uniform noise (seed 7), energy+mass "
@@ -57,25 +79,25 @@ def _peaks():
 
 
 def _sources_sha256():
-    """Hashes of the sources the timed step kernel (k_step) is built from."""
+    """Hashes of the sources the timed step kernel (k_step2) is built from."""
     out = {}
-    for name in ("lb_fp32.cu", "lb_device.cuh", "lb_internal.h"):
+    for name in ("lb_pair.cu", "lb_packed.cuh", "lb_device.cuh", "lb_internal.h"):
         path = os.path.join(ROOT, "paper_1008_2865_gb300", "csrc", name)
         with open(path, "rb") as fh:
             out[name] = hashlib.sha256(fh.read()).hexdigest()
     return out
 
 
-def _traffic_record(nx, ny, launch):
-    """DRAM bytes per launch of the step kernel from the committed ncu summary, if the
-    kernel sources and launch shape are unchanged since it was taken (else None)."""
+def _traffic_record(nx, ny):
+    """DRAM bytes per step of the step kernel from the committed ncu summary, if the kernel
+    sources are unchanged since it was taken (else None)."""
     rec_path = os.path.join(ROOT, "profiles", "step_fp32_traffic.json")
     try:
         with open(rec_path) as fh:
             rec = json.load(fh)
         if (rec.get("sources_sha256") == _sources_sha256() and rec.get("nx") == nx
-                and rec.get("ny") == ny and list(rec.get("launch", [])) == list(launch)):
-            return float(rec["dram_bytes_per_launch"])
+                and rec.get("ny") == ny):
+            return float(rec["dram_bytes_per_launch"]) / rec["steps_per_launch"]
     except Exception:
         pass
     return None
@@ -182,7 +204,7 @@ def run_batched(steps, warmup, stream, dev):
             "one_by_one_mlups": sites * steps / (ms_seq / 1e3) / 1e6,
             "speedup_vs_one_by_one": ms_seq / ms_batch,
             "launch": {"block_x": launch[0], "rows_per_cta": launch[1], "cuda_graph": bool(launch[2])},
-            "launches_per_step": "1 (+1 per-replica reduction every 10 steps)"}
+            "launches_per_step": "1 per two steps (+2 per trace row)"}
 
 
 def run_adjoint(stream, dev, T=2000, n=512):
@@ -229,8 +251,8 @@ def run_adjoint(stream, dev, T=2000, n=512):
 
 def run_fp16(steps, warmup, stream, dev, peak):
     """The same 8192^2 workload with the populations stored as FP16 deviations (44 B per
-    site: 18 B read + 18 B written + 4 + 4 B of psi), FP32 arithmetic: device-resident
-    MLUPS and the fraction of the copy bandwidth at 44 B/site."""
+    site and pass of two steps: 18 B read + 18 B written + 4 + 4 B of psi), FP32 arithmetic:
+    device-resident MLUPS and the fraction of the copy bandwidth."""
     import torch
 
     from paper_1008_2865_gb300 import Lattice, inputs, tune
@@ -254,27 +276,28 @@ def run_fp16(steps, warmup, stream, dev, peak):
         e = lat.energy()
         if not all(np.isfinite(e)):
             raise RuntimeError(f"non-finite FP16-storage energies {e}")
-    gbs = 44 * NX * NY / (ms / 1e3) / 1e9
+    per_site = bytes_per_site_step("fp16_delta", launch[2] == 1)
+    gbs = per_site * NX * NY / (ms / 1e3) / 1e9
     return {"workload": WORKLOAD.format(n=NX).replace("FP32 (deviation storage)",
                                                       "FP16 deviation storage, FP32 arithmetic"),
             "mlups": NX * NY / (ms / 1e3) / 1e6, "ms_per_step": ms, "steps": steps,
             "launch": {"block_x": launch[0], "rows_per_cta": launch[1],
                        "pipeline": ["register-prefetch", "bulk-copy rings"][launch[2]]},
-            "roofline": {"bound": "hbm", "bytes_per_site": 44, "achieved": gbs, "peak": peak,
+            "roofline": {"bound": "issue", "bytes_per_site": per_site, "achieved": gbs, "peak": peak,
                          "unit": "GB/s", "frac": gbs / peak,
-                         "roof_mlups": peak * 1e9 / 44 / 1e6}}
+                         "roof_mlups": peak * 1e9 / per_site / 1e6}}
 
 
 def run_step_split(stream, dev, launch, steps=20):
-    """Time of a plain step and of a step with the fused energy/mass reduction, each
-    timed over `steps` consecutive steps of the 8192^2 FP32 lattice (trace_every = 0
-    and 1), with the benchmark's launch shape."""
+    """Time of a plain step and of a step with a trace row (energies and mass) of the
+    8192^2 FP32 lattice with the benchmark's launch shape: trace_every = 0, and what a
+    period of two takes beyond its plain step."""
     import torch
 
     from paper_1008_2865_gb300 import Lattice, inputs
     rho0 = inputs.noisy_density(NX, NY, SEED, mean=0.7, amp=0.01, mode="rel")
     out = {}
-    for name, te in (("plain", 0), ("reduce", 1)):
+    for name, te in (("plain", 0), ("reduce", 2)):
         with Lattice(rho0, omega=OMEGA, G1=G1, G2=G2, trace_every=te, device=dev,
                      stream=stream.cuda_stream) as lat:
             lat.set_launch(*launch)
@@ -287,6 +310,7 @@ def run_step_split(stream, dev, launch, steps=20):
             e1.record(stream)
             e1.synchronize()
             out[name + "_ms"] = e0.elapsed_time(e1) / steps
+    out["reduce_ms"] = 2 * out["reduce_ms"] - out["plain_ms"]
     out["reduce_over_plain"] = out["reduce_ms"] / out["plain_ms"]
     return out
 
@@ -403,9 +427,9 @@ def run_ours(args):
     value = N * args.steps * ws / (ms_max / 1e3) / 1e6
     per_launch_s = ms / 1e3 / args.steps
     peak, peak_src = _peaks()
-    achieved = (BYTES_PER_SITE if args.prec == "fp32" else 44) * N / per_launch_s / 1e9
-    traffic = _traffic_record(NX, NY, launch)
-    bytes_per_site = BYTES_PER_SITE if args.prec == "fp32" else 44
+    bytes_per_site = bytes_per_site_step(args.prec, launch[2] == 1)
+    achieved = bytes_per_site * N / per_launch_s / 1e9
+    traffic = _traffic_record(NX, NY) if launch[2] == 0 and args.prec == "fp32" else None
 
     if args.skip_e2e:
         print(json.dumps({"size": NX, "prec": args.prec, "launch": launch, "MLUPS": value,
@@ -455,8 +479,8 @@ def run_ours(args):
                          "frac": achieved / peak, "traffic": traffic,
                          "peak_source": peak_src,
                          "kernel": ("k_step_bulk (one launch per step)" if launch[2] else
-                                    "k_step (one launch per step; a reduction step adds "
-                                    "k_step_total, its grid sum)"),
+                                    "k_step2 (two steps per launch; a trace row adds "
+                                    "k_trace_partial and k_trace_total)"),
                          "bytes_per_site": bytes_per_site},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": "MLUPS",
@@ -465,9 +489,7 @@ def run_ours(args):
                     "includes": "lb_init from pinned host rho (H2D), lb_step(K), lb_trace of the "
                                 "K/10 trace rows (t, mass, E_s, E_m, E_bulk) (D2H), lb_fields rho "
                                 "to pinned host (D2H)"},
-            # one step kernel per step; the register-prefetch pipeline's reduction steps
-            # (t % TRACE_EVERY == 0; the timed region starts at such a t) add k_step_total
-            "gpu_launches": args.steps + (0 if launch[2] else -(-args.steps // TRACE_EVERY)),
+            "gpu_launches": (args.steps if launch[2] else step_launches(args.steps)),
             "clocks": clocks,
             "batched": batched,
             "adjoint": adjoint,

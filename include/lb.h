@@ -230,13 +230,14 @@ lb_status lb_adjoint(lb_state* s, long steps, const double* rho_target, int chec
  * LB_ERR_CUDA, LB_ERR_NONFINITE. */
 lb_status lb_objective(lb_state* s, const double* rho_target, double* J);
 
-/* ---- Batches: many independent lattices advanced by one launch per step ----
+/* ---- Batches: many independent lattices advanced together ----
  * A batch holds `count` replicas (each with its own size, couplings, omega,
  * rho_ref and initial density; all with the same prec — LB_FP32 or
  * LB_FP16_DELTA —, trace_every and device), e.g. a G2 sweep with distinct
- * seeds. lb_batch_step advances all of them: one persistent launch per step
- * strides over a work list of every replica's tiles, and steps are replayed
- * from a CUDA graph of one trace period when the batch time is aligned to it.
+ * seeds. lb_batch_step advances all of them: one persistent launch per two steps
+ * (one, where a step is left over) strides over a work list of every replica's
+ * tiles, and steps are replayed from a CUDA graph of one trace period when the
+ * batch time is aligned to it.
  * A replica's fields, energies and trace are bit-identical to those of the
  * same lattice run alone with the same launch shape (register-prefetch
  * pipeline). The paper runs its A2 scan (Sec. 4) as separate simulations;

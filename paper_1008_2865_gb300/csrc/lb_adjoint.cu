@@ -930,11 +930,15 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
     double2* sums = reinterpret_cast<double2*>(reinterpret_cast<char*>(scr) + word_bytes);
     double2* tot = sums + (size_t)grid * (size_t)(rows + 1);
     float* terms = reinterpret_cast<float*>(tot + (rows + 1));
-    auto add_terms = [&](long long n) -> bool {
-        k_adj_sums<<<dim3(grid, (unsigned)n), kAdjThreads, 0, st>>>(terms, N, sums);
-        if (cudaGetLastError() != cudaSuccess) return false;
-        k_adj_sums_total<<<(unsigned)n, kAdjThreads, 0, st>>>(sums, grid, tot, cnt, acc + 4);
-        return cudaGetLastError() == cudaSuccess;
+    auto add_terms = [&](int n) -> bool {
+        for (int r = 0; r < n; r += 32768) {      // within the grid's limit in y
+            const int m = n - r < 32768 ? n - r : 32768;
+            k_adj_sums<<<dim3(grid, m), kAdjThreads, 0, st>>>(terms + (size_t)2 * N * r, N, sums);
+            if (cudaGetLastError() != cudaSuccess) return false;
+            k_adj_sums_total<<<m, kAdjThreads, 0, st>>>(sums, grid, tot, cnt, acc + 4);
+            if (cudaGetLastError() != cudaSuccess) return false;
+        }
+        return true;
     };
     int in4 = 0;             // lam4[in4] holds the adjoint
     if (held) {

@@ -1,8 +1,8 @@
 // lb_batch.cu — the lb_batch_* entry points of include/lb.h: many independent
 // lattices (replicas of possibly different sizes and couplings, e.g. a G2
-// sweep with distinct seeds) advanced together, one launch per step over a
-// work list of all replicas' tiles (k_step_batch in lb_fp32.cu), replayed
-// from a CUDA graph of one trace period. Each replica is an lb_state, so
+// sweep with distinct seeds) advanced together, one launch per two steps over a
+// work list of all replicas' tiles (k_step2_batch in lb_pair.cu; k_step_batch in
+// lb_fp32.cu where a step is left over), replayed from a CUDA graph of one trace period. Each replica is an lb_state, so
 // energies, fields and traces reuse the single-lattice code.
 #include <algorithm>
 #include <new>

@@ -7,8 +7,8 @@
 // the kernel then is instruction issue (63% of the slots busy, 5.2 TB/s of HBM
 // traffic at 4096^2), so every thread works on two adjacent columns with packed FP32
 // instructions (lb_packed.cuh): about 190 instructions per site and step, halo
-// included, against 343 of k_step. 8192^2, us per plain step: FP32 827 -> 493,
-// FP16 717 -> 451; 2050x1999 63.7 -> 37.8; 1024^2 20.5 -> 14.4.
+// included, against 343 of k_step. 8192^2, us per plain step: FP32 827 -> 495,
+// FP16 717 -> 445; 2050x1999 63.7 -> 37.9; 1024^2 20.5 -> 14.4.
 //
 // A CTA of TH threads owns 2 TH - 8 output columns (two steps need a halo of four
 // collision columns on each side) and marches down its rows. Iteration r: stage 1
@@ -20,11 +20,17 @@
 // they are summed as the speeds arrive, and a row waits in shared memory as three
 // values per site instead of nine (496 against 524 us per FP32 step at 8192^2).
 //
-// Measured and not kept, us per FP32 step at 8192^2: strips of 248 columns (TH = 128)
-// 515-536; 16 instead of 12 resident FP32 warps per SM, at 128 registers with 12 bytes
-// spilled, 551 (FP16 fits 128 without spills and gains 4%); populations unpacked or
-// loaded later than at the top of the iteration 568; without the L2 prefetch of the
-// population rows 619 (with an earlier form of the rest).
+// Measured and not kept, us per step at 8192^2 (FP32 / FP16; 498 / 445 as it is): strips of
+// 184 and 248 columns (TH = 96, 128) 502 / 481 and 517 / 472; 16 instead of 12 resident
+// FP32 warps per SM, at 128 registers with 12 bytes spilled, 551 (FP16 fits 128 without
+// spills and gains 4%); populations unpacked or loaded later than at the top of the
+// iteration 568; the rings' first rows repeated behind the last, so that a stencil is
+// one base address, 500 / 456; the row loop unrolled by two 498 / 505; dpsi rows loaded
+// an iteration earlier 504 / 498; streaming loads 534 / 449, stores 495 / 449; without the
+// L2 prefetch of the population rows 619 (with an earlier form of the rest). Stage 1 alone,
+// streamed into the output, as a single step of its own: 920 / 523, and 16.5 at 1024^2
+// against 14.4. In a narrow last strip the second warp only keeping the barriers:
+// 96-replica batch 192 against 178.
 //
 // Every site's arithmetic is that of k_step, operation by operation, so the fields
 // are bit-identical to two single steps. If state t has a trace row, stage 1 leaves its

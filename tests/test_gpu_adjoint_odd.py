@@ -51,3 +51,16 @@ def test_held_reverse_equals_the_two_passes(nx, ny):
     assert np.linalg.norm(g - gt) <= 1e-4 * np.linalg.norm(gt)
     for k in range(2):
         assert abs(gG[k] - gGt[k]) <= 1e-4 * abs(gGt[k])
+
+
+def test_held_segment_of_more_steps_than_a_grid_dimension():
+    """One segment of 70,000 steps (more than a grid may have rows) against segments of
+    265: the same bits. The lattice has no unstable mode, so nothing overflows."""
+    r0 = inputs.noisy_density(5, 5, 11, mean=0.7, amp=0.01, mode="rel")
+    tgt = inputs.noisy_density(5, 5, 12, mean=0.7, amp=0.01, mode="rel")
+    got = []
+    for every in (0, 70000):
+        with Lattice(r0, G1=-3.0, G2=0.2, trace_every=0) as lat:
+            got.append(lat.adjoint(70000, tgt, checkpoint_every=every))
+    assert got[0][0] == got[1][0] and got[0][2] == got[1][2]
+    assert np.array_equal(got[0][1], got[1][1])
