@@ -30,7 +30,8 @@
 // L2 prefetch of the population rows 619 (with an earlier form of the rest). Stage 1 alone,
 // streamed into the output, as a single step of its own: 920 / 523, and 16.5 at 1024^2
 // against 14.4. In a narrow last strip the second warp only keeping the barriers:
-// 96-replica batch 192 against 178.
+// 96-replica batch 192 against 178. Odd nx with the test for split pairs only in the strips
+// at the periodic edge, two bodies in one kernel: 46.1 against 41.0 at 2051x1999.
 //
 // Every site's arithmetic is that of k_step, operation by operation, so the fields
 // are bit-identical to two single steps. If state t has a trace row, stage 1 leaves its
@@ -522,9 +523,10 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
 }
 
 // Resident threads per SM the registers are cut for: 16 warps where the kernel fits
-// 128 registers without spilling (FP16, omega = 1), otherwise 12.
+// 128 registers (FP16; with omega != 1 8 bytes are spilled, 494 us per step at 8192^2
+// against 522-549 with 12 warps), otherwise 12.
 template <typename T, bool OM1>
-constexpr int kPairThreads = OM1 && sizeof(T) == 2 ? 512 : 384;
+constexpr int kPairThreads = sizeof(T) == 2 ? 512 : 384;
 constexpr int kTH = 64;   // threads per CTA
 
 template <typename T, int TH, bool OM1, bool ODD, bool TRACE>
