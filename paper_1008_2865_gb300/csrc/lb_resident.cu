@@ -7,7 +7,7 @@
 // memory from step to step: a step is one collision of all the tile's sites at once, a
 // barrier, one streaming. Only the sites next to a tile's edge go through L2. us per
 // step, before -> after: 70x45 10.8 -> 1.9, 128^2 8.2 -> 1.8, 250x187 10.1 -> 2.3, 512^2
-// 10.3 -> 4.3.
+// 10.3 -> 4.1.
 //
 // What a step costs now: two passes over the tile at about 0.4 us each (128^2) and the
 // halo's way to L2 and back, 0.5 us. The halo is one ring of moments (with omega = 1 a
@@ -36,7 +36,10 @@ namespace {
 
 using namespace dev;
 
-constexpr int kResThreads = 768;   // at most
+// Threads at most, by the registers (us per step at 512^2 / 600^2 with 768, 896 and 1024
+// threads: 4.25 / 5.32, 4.11 / 5.11, 4.26 / 5.30)
+template <bool OM1>
+constexpr int kResThreads = OM1 ? 896 : 768;
 
 template <typename T>
 struct ResArgs {
@@ -87,7 +90,7 @@ __device__ __forceinline__ float2 stored2<__half>(float2 v)
 }
 
 template <typename T, bool OM1>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(const ResArgs<T> A)
+__global__ void __launch_bounds__(kResThreads<OM1>, 1) k_resident(const ResArgs<T> A)
 {
     const int nt = blockDim.x;
     extern __shared__ __align__(16) float sm[];
@@ -382,13 +385,14 @@ cudaError_t resident_launch(const StepArgs<T>& a, ResidentBuf& b, int steps, flo
     b.tag += (unsigned)steps;
     const bool om1 = a.omega == 1.0f;
     const size_t smem = res_smem(b.tw, b.th, om1);
-    // a thread per collision pair and per halo word, 256 to 768 (us per step, 256 / 384 /
+    // a thread per collision pair and per halo word, from 256 on (us per step, 256 / 384 /
     // 512 / 768 threads: 128^2 1.80 / 1.81 / 1.86 / 1.96, 250x187 2.49 / 2.31 / 2.36 / 2.48,
     // 512^2 5.43 / 4.47 / 4.48 / 4.28)
     const int pairs = (b.tw + 4) / 2 * (b.th + 2);
     const int words = halo_psi(b.tw, b.th) + (om1 ? 1 : 3) * halo_mom(b.tw, b.th);
     int threads = ((pairs > words ? pairs : words) + 31) / 32 * 32;
-    threads = threads < 256 ? 256 : threads > kResThreads ? kResThreads : threads;
+    const int most = om1 ? kResThreads<true> : kResThreads<false>;
+    threads = threads < 256 ? 256 : threads > most ? most : threads;
     return om1 ? launch_resident<T, true>(A, b.gx * b.gy, threads, smem, s)
                : launch_resident<T, false>(A, b.gx * b.gy, threads, smem, s);
 }
