@@ -686,7 +686,7 @@ bool reverse_plan(int nx, int ny, int num_sms, RevArgs& R, int& tiles)
         for (int gy = 1; gy <= num_sms / gx; ++gy) {
             const int th = (ny + gy - 1) / gy;
             if ((ny + th - 1) / th != gy || (tw * th < 64 && gx * gy > 1)) continue;
-            if (4 * (size_t)rev_floats(tw, th) > 226 * 1024) continue;
+            if (4 * (size_t)rev_floats(tw, th) > kHeldSmem) continue;
             const double cost = (tw + 4) * (th + 4) + 0.5 * tw * th;
             if (cost < best) {
                 best = cost;
@@ -952,8 +952,9 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
         const int sites = (R.tw + 4) * (R.th + 4);
         int threads = (sites + 31) / 32 * 32;
         threads = threads < 256 ? 256 : threads > kRevThreads ? kRevThreads : threads;
+        // the limit, not this launch's size: another thread may be launching another lattice
         if (cudaFuncSetAttribute(k_adj_reverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
+                                 kHeldSmem) != cudaSuccess)
             return fail();
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(rev_tiles);

@@ -211,6 +211,9 @@ template <typename T>
 cudaError_t batch_trace_partials(const BatchLaunch<T>& b, cudaStream_t s);
 template <typename T>
 cudaError_t batch_reduce(const BatchLaunch<T>& b, cudaStream_t s);
+// Shared memory per CTA of the kernels that hold a lattice on the SMs (227 KB at most, less
+// their static words).
+constexpr int kHeldSmem = 226 * 1024;
 // Many steps of a small lattice in one launch (lb_resident.cu): the tiles its CTAs hold
 // and the buffers they exchange through.
 struct ResidentBuf {

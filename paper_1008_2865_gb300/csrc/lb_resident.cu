@@ -347,8 +347,9 @@ __global__ void __launch_bounds__(kResThreads<OM1>, 1) k_resident(const ResArgs<
 template <typename T, bool OM1>
 cudaError_t launch_resident(const ResArgs<T>& A, int grid, int threads, size_t smem, cudaStream_t s)
 {
+    // the limit, not this launch's size: another thread may be launching another lattice
     cudaError_t e = cudaFuncSetAttribute(k_resident<T, OM1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         kHeldSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
@@ -435,7 +436,7 @@ bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b)
         for (int gy = 1; gy <= num_sms / gx; ++gy) {
             const int th = (ny + gy - 1) / gy;
             if ((ny + th - 1) / th != gy) continue;
-            if (res_smem(tw, th, om1) > 226 * 1024) continue;
+            if (res_smem(tw, th, om1) > kHeldSmem) continue;
             if (tw * th < 64 && gx * gy > 1) continue;
             const double cost = (tw + 4) / 2 * (th + 2) + 0.5 * tw * th / 2 + 0.5 * halo_psi(tw, th);
             if (cost < best) {

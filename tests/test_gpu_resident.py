@@ -92,3 +92,47 @@ def test_captured_steps_replay(nx):
             g.replay()
         torch.cuda.synchronize()
         _same(ref, lat.fields())
+
+
+def test_held_lattices_on_streams_of_their_own_threads():
+    """Lattices of different sizes (so different tiles and shared memory), and an adjoint,
+    each stepped by its own thread on its own stream at the same time, against the same
+    work one after another."""
+    import threading
+
+    import torch
+    from paper_1008_2865_gb300 import Lattice, inputs
+    jobs = [(512, 384, 0), (96, 80, 0), (300, 301, 0), (128, 128, 40)]
+
+    def work(nx, ny, adjoint, stream):
+        rho0 = inputs.noisy_density(nx, ny, seed=nx, mean=0.7, amp=0.01, mode="rel")
+        out = []
+        for _ in range(6):
+            with Lattice(rho0, G1=-5.0, G2=0.6, trace_every=7, stream=stream) as lat:
+                if adjoint:
+                    J, g, gG = lat.adjoint(adjoint, np.ascontiguousarray(rho0[::-1]))
+                    out += [np.array([J, *gG]), g]
+                else:
+                    for _ in range(5):
+                        lat.step(20)
+                out += [*lat.fields(), lat.trace()]
+        return out
+
+    ref = [work(*j, 0) for j in jobs]
+    got, bad = [None] * len(jobs), []
+
+    def run(i):
+        try:
+            s = torch.cuda.Stream()
+            got[i] = work(*jobs[i], s.cuda_stream)
+        except Exception as exc:      # shown by the main thread
+            bad.append((i, exc))
+
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
+    for one, two in zip(ref, got):
+        _same(one, two)
