@@ -234,9 +234,9 @@ void free_state(lb_state* s)
     delete s;
 }
 
-// Steps of a small lattice that stay on the SMs (lb_resident.cu): from two steps on,
-// as many per launch as the trace rows they append can be kept.
-lb_status step_resident(lb_state* s, long n)
+// Steps of a small lattice that stay on the SMs (lb_resident.cu), as many per launch as the
+// trace rows they append can be kept.
+lb_status step_held(lb_state* s, long n)
 {
     ResidentBuf& b = s->res_buf;
     while (n > 0) {
@@ -248,6 +248,7 @@ lb_status step_resident(lb_state* s, long n)
             if (m > room) m = (long)room;
         }
         if (m > (1L << 20)) m = 1L << 20;
+        if (s->in_graphs && m % 2 == 0) --m;   // a launch swaps the buffers once
         const cudaError_t e =
             s->p.prec == LB_FP32
                 ? fp32_resident(make_args<float>(s), b, s->launch.block_x, (int)m, s->stream)
@@ -273,39 +274,48 @@ cudaError_t pair_step(lb_state* s, bool traced)
     return trace_rows<T>(a, r, s->stream);
 }
 
+// n steps in launches of their own or (`pairs`) two at a time (lb_pair.cu): the same
+// fields bit for bit, half the memory traffic.
+lb_status step_streamed(lb_state* s, long n, bool pairs)
+{
+    const int te = s->p.trace_every;
+    const bool bulk = s->launch.pipeline == 1;
+    pairs = pairs && pairs_pay(s->N);
+    // one pair fewer if the buffers would not swap as single steps swap them
+    int singles = pairs && s->in_graphs && pairs_made(s->t, n, te) % 2 != 0 ? 2 : 0;
+    while (n > 0) {
+        const bool reduce = te > 0 && s->t % te == 0;
+        bool pair = pairs && pair_at(s->t, n, te);
+        if (singles == 1 || (singles == 2 && pair)) {
+            --singles;
+            pair = false;
+        }
+        cudaError_t e;
+        if (s->p.prec == LB_FP32)
+            e = pair   ? pair_step<float>(s, reduce)
+                : bulk ? fp32_step_bulk(make_args<float>(s), s->launch, reduce, s->stream)
+                       : fp32_step(make_args<float>(s), s->launch, reduce, s->stream);
+        else
+            e = pair   ? pair_step<__half>(s, reduce)
+                : bulk ? fp16_step_bulk(make_args<__half>(s), s->launch, reduce, s->stream)
+                       : fp16_step(make_args<__half>(s), s->launch, reduce, s->stream);
+        if (e != cudaSuccess) return fail_cuda(s);
+        s->cur ^= 1;
+        s->t += pair ? 2 : 1;
+        n -= pair ? 2 : 1;
+    }
+    return LB_OK;
+}
+
 lb_status step_fp32(lb_state* s, long n)
 {
     // in a stream capture every step is a launch of its own, so that a graph of an even
     // number of steps can be replayed: each step swaps the buffers once
-    const bool many = n >= 2 && s->launch.pipeline == 0 && !stream_captures(s->stream);
-    if (many && s->res_buf.gx > 0) return step_resident(s, n);
-    for (long k = 0; k < n; ++k) {
-        const bool reduce = s->p.trace_every > 0 && (s->t % s->p.trace_every) == 0;
-        cudaError_t e;
-        const bool bulk = s->launch.pipeline == 1;
-        // two steps go through the lattice together (lb_pair.cu) unless the second state
-        // has a trace row: the same fields bit for bit, half the memory traffic
-        const bool next_reduces =
-            s->p.trace_every > 0 && ((s->t + 1) % s->p.trace_every) == 0;
-        if (many && !next_reduces && k + 1 < n && pairs_pay(s->N)) {
-            e = s->p.prec == LB_FP32 ? pair_step<float>(s, reduce) : pair_step<__half>(s, reduce);
-            if (e != cudaSuccess) return fail_cuda(s);
-            s->cur ^= 1;
-            s->t += 2;
-            ++k;
-            continue;
-        }
-        if (s->p.prec == LB_FP32)
-            e = bulk ? fp32_step_bulk(make_args<float>(s), s->launch, reduce, s->stream)
-                     : fp32_step(make_args<float>(s), s->launch, reduce, s->stream);
-        else
-            e = bulk ? fp16_step_bulk(make_args<__half>(s), s->launch, reduce, s->stream)
-                     : fp16_step(make_args<__half>(s), s->launch, reduce, s->stream);
-        if (e != cudaSuccess) return fail_cuda(s);
-        s->cur ^= 1;
-        s->t += 1;
-    }
-    return LB_OK;
+    const bool captures = stream_captures(s->stream);
+    s->in_graphs = s->in_graphs || (captures && n > 0);
+    const bool many = n >= 2 && s->launch.pipeline == 0 && !captures;
+    if (many && s->res_buf.gx > 0) return step_held(s, n);
+    return step_streamed(s, n, many);
 }
 
 }  // namespace

@@ -26,6 +26,7 @@ struct lb_batch {
     long long t = 0;
     int cur = 0;
     bool poisoned = false;
+    bool in_graphs = false;         // as in lb_state
     // device tables
     void* d_args[2] = {nullptr, nullptr};   // StepArgs<T>[nreps] for buffers 0 and 1
     int4* d_tiles = nullptr;
@@ -168,17 +169,13 @@ cudaError_t enqueue_pair(const lb_batch* b, cudaStream_t s, int cur, bool traced
     return e;
 }
 
-// Enqueue step t (buffers `cur` in) of every replica on stream s, or (`pairs`) steps t and
-// t + 1 together when `left` allows and state t + 1 has no trace row; returns through `taken`
-// how many steps that was. Either way the buffers swap once.
-cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cur, long long left,
-                          bool pairs, int& taken)
+// Enqueue step t (buffers `cur` in) of every replica on stream s, or (`pair`) steps t and
+// t + 1 together. Either way the buffers swap once.
+cudaError_t enqueue_steps(const lb_batch* b, cudaStream_t s, long long t, int cur, bool pair)
 {
     const int te = b->trace_every;
     const bool reduce = te > 0 && t % te == 0;
-    const bool next_reduces = te > 0 && (t + 1) % te == 0;
-    taken = pairs && !next_reduces && left >= 2 ? 2 : 1;
-    if (taken == 2)
+    if (pair)
         return b->prec == LB_FP32 ? enqueue_pair<float>(b, s, cur, reduce)
                                   : enqueue_pair<__half>(b, s, cur, reduce);
     return b->prec == LB_FP32 ? fp32_batch_step(batch_launch<float>(b, cur), reduce, s)
@@ -196,8 +193,10 @@ bool build_graph(lb_batch* b, int cur)
     }
     cudaError_t e = cudaSuccess;
     int in = cur;
-    for (int k = 0, taken = 0; k < b->period && e == cudaSuccess; k += taken) {
-        e = enqueue_steps(b, b->cap, k, in, b->period - k, true, taken);
+    for (int k = 0; k < b->period && e == cudaSuccess;) {
+        const bool pair = pair_at(k, b->period - k, b->trace_every);
+        e = enqueue_steps(b, b->cap, k, in, pair);
+        k += pair ? 2 : 1;
         in ^= 1;
     }
     cudaGraph_t g = nullptr;
@@ -291,22 +290,28 @@ lb_status lb_batch_step(lb_batch* b, long n)
     if (b->poisoned) return LB_ERR_STATE;
     DeviceScope dev(b->device);
     if (!dev.ok) return poison(b);
-    // in a caller's capture every step is a launch of its own and swaps the buffers once
+    // in a caller's capture every step is a launch of its own and swaps the buffers once;
+    // from then on as many pairs are taken as swap the buffers alike, without the period's graph
     const bool captures = stream_captures(b->stream);
+    b->in_graphs = b->in_graphs || (captures && n > 0);
+    int singles = b->in_graphs && pairs_made(b->t, n, b->trace_every) % 2 != 0 ? 2 : 0;
     while (n > 0) {
-        if (b->use_graph && !captures && b->period > 0 && b->t % b->period == 0 && n >= b->period &&
-            build_graph(b, b->cur)) {
+        if (b->use_graph && !b->in_graphs && b->period > 0 && b->t % b->period == 0 &&
+            n >= b->period && build_graph(b, b->cur)) {
             if (cudaGraphLaunch(b->exec[b->cur], b->stream) != cudaSuccess) return poison(b);
             b->t += b->period;
             n -= b->period;
             b->cur ^= b->period_flips;
         } else {
-            int taken = 1;
-            if (enqueue_steps(b, b->stream, b->t, b->cur, n, !captures, taken) != cudaSuccess)
-                return poison(b);
-            b->t += taken;
+            bool pair = !captures && pair_at(b->t, n, b->trace_every);
+            if (singles == 1 || (singles == 2 && pair)) {
+                --singles;
+                pair = false;
+            }
+            if (enqueue_steps(b, b->stream, b->t, b->cur, pair) != cudaSuccess) return poison(b);
+            b->t += pair ? 2 : 1;
             b->cur ^= 1;
-            n -= taken;
+            n -= pair ? 2 : 1;
         }
     }
     for (lb_state* s : b->reps) {

@@ -306,6 +306,7 @@ struct lb_state {
     long long wait_cycles = 2000000000LL;
     int skip_unit0 = 0;            // test hook of lb_set_wait_limit
     lbsc::ResidentBuf res_buf;     // small lattices: tiles held on the SMs over many steps
+    bool in_graphs = false;        // steps were captured: n steps swap the buffers as n single ones do
     // FP64 parity storage
     double* f64[2] = {nullptr, nullptr};
     double* psi64 = nullptr;
@@ -340,6 +341,26 @@ void* state_alloc(lb_state* s, size_t bytes);
 }  // namespace lbsc
 
 namespace lbsc {
+// Whether steps t and t + 1 go through a lattice or batch together when `left` steps are
+// left: not when state t + 1 has a trace row (every te steps; 0: none).
+inline bool pair_at(long long t, long long left, int te)
+{
+    return left >= 2 && !(te > 0 && (t + 1) % te == 0);
+}
+// How many pairs n steps from t make. A captured graph reads and writes the buffers that
+// were in place when it was captured, and its replays are valid after any number of further
+// steps that swaps the buffers as often, modulo two, as single steps do: once each. A pair swaps
+// them once for two steps, so states whose steps have been captured take an even number of pairs.
+inline long long pairs_made(long long t, long long n, int te)
+{
+    long long pairs = 0;
+    for (long long k = 0; k < n;) {
+        const bool pair = pair_at(t + k, n - k, te);
+        pairs += pair;
+        k += pair ? 2 : 1;
+    }
+    return pairs;
+}
 // Take n steps of an FP32 or FP16 state, several per launch where that pays (lb_step).
 lb_status advance_delta(lb_state* s, long n);
 template <typename T>
