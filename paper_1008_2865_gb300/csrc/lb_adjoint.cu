@@ -600,12 +600,12 @@ __global__ void __launch_bounds__(kRevThreads, 1) k_adj_reverse(const RevArgs R)
             }
         }
         if (last) return;
-        long long t_end = 0;
+        long long t_first = 0;
         unsigned polls = 0;
         for (int q = tid; q < nl; q += nt) {
             const int2 e = hl[q];
             uint4 v = get_word(words + e.y);
-            while (v.w != tag && !wait_over(a, &s_fail, polls, t_end)) v = get_word(words + e.y);
+            while (v.w != tag && !wait_over(a, &s_fail, polls, t_first)) v = get_word(words + e.y);
             float* l = L + e.x;
             l[0] = __uint_as_float(v.x);
             l[LS] = __uint_as_float(v.y);

@@ -323,12 +323,12 @@ __device__ __forceinline__ uint4 get_word(const uint4* p)
 // wait limit has passed or another CTA has given up flags the state and the CTA (*fail).
 template <typename T>
 __device__ __forceinline__ bool wait_over(const StepArgs<T>& a, int* fail, unsigned& polls,
-                                          long long& t_end)
+                                          long long& t_first)
 {
     if ((++polls & 255u) == 0) {
         const long long now = clock64();
-        if (t_end == 0) t_end = now + a.wait_cycles;
-        if (now > t_end || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
+        if (t_first == 0) t_first = now;
+        if (limit_passed(t_first, now, a.wait_cycles) || (*reinterpret_cast<volatile int*>(a.err) & 1)) {
             atomicOr(a.err, 1);
             *reinterpret_cast<volatile int*>(fail) = 1;
         }

@@ -62,6 +62,13 @@ inline bool stream_captures(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
+// Whether a wait that began at clock `first` has lasted longer than `limit` cycles at `now`.
+// (The difference, not first + limit, which a limit near the type's largest overflows.)
+__host__ __device__ inline bool limit_passed(long long first, long long now, long long limit)
+{
+    return now - first > limit;
+}
+
 constexpr int kTraceCap = 65536;     // rows kept in the device trace ring
 constexpr int kTraceCols = 5;        // (t, mass, E_s, E_m, E_bulk)
 

@@ -316,9 +316,9 @@ __global__ void __launch_bounds__(kResThreads<OM1>, 1) k_resident(const ResArgs<
         // ---- collisions that need no halo, while the neighbours' values arrive
         traced = is_traced(s + 1);
         collide(0, nfree, traced);
-        long long t_end = 0;
+        long long t_first = 0;
         unsigned polls = 0;
-        auto give_up = [&]() { return wait_over(a, &s_fail, polls, t_end); };
+        auto give_up = [&]() { return wait_over(a, &s_fail, polls, t_first); };
         for (int q = tid; q < nm * kQuads<OM1> + np; q += nt) {
             if (q < nm * kQuads<OM1>) {
                 const int u = OM1 ? 0 : q / nm;
