@@ -17,30 +17,47 @@ namespace lbsc {
 // Test hook: allocations left before one is made to fail (-1: never).
 static std::atomic<int> g_fail_allocs_after{-1};
 
-void* state_alloc(lb_state* s, size_t bytes)
+bool state_alloc(lb_state* s, const std::vector<Buffer>& buffers)
 {
-    {
+    size_t total = 0;
+    for (const Buffer& b : buffers) {
         int left = g_fail_allocs_after.load();
         while (left >= 0 && !g_fail_allocs_after.compare_exchange_weak(left, left - 1)) {
         }
-        if (left == 0) return nullptr;   // the hook's failure (counter is now -1: disarmed)
+        if (left == 0) return false;   // the hook's failure (counter is now -1: disarmed)
+        total += guarded_size(b.bytes) + 2 * kGuardBytes;
     }
-    // round the usable size up so the tail guard starts 256-byte aligned
-    const size_t body = (bytes + kGuardBytes - 1) / kGuardBytes * kGuardBytes;
-    void* base = nullptr;
-    if (cudaMalloc(&base, body + 2 * kGuardBytes) != cudaSuccess) {
+    void* block = nullptr;
+    if (cudaMalloc(&block, total) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return false;
     }
-    char* b = static_cast<char*>(base);
-    if (cudaMemsetAsync(b, kGuardByte, kGuardBytes, s->stream) != cudaSuccess ||
-        cudaMemsetAsync(b + kGuardBytes + body, kGuardByte, kGuardBytes, s->stream) != cudaSuccess) {
+    // the guards: one fill over small buffers and all, otherwise one at each end and where
+    // two buffers meet
+    char* at = static_cast<char*>(block);
+    bool ok = true;
+    auto fill = [&](char* p, size_t n) {
+        ok = ok && cudaMemsetAsync(p, kGuardByte, n, s->stream) == cudaSuccess;
+    };
+    const bool small = total <= (64u << 10);
+    fill(at, small ? total : kGuardBytes);
+    const size_t had = s->allocs.size();
+    for (size_t k = 0; k < buffers.size(); ++k) {
+        const size_t body = guarded_size(buffers[k].bytes);
+        *buffers[k].ptr = at + kGuardBytes;
+        s->allocs.push_back({at, body});
+        if (!small) fill(at + kGuardBytes + body, (k + 1 < buffers.size() ? 2 : 1) * kGuardBytes);
+        at += body + 2 * kGuardBytes;
+    }
+    if (!ok) {
         cudaGetLastError();
-        cudaFree(base);
-        return nullptr;
+        cudaFree(block);
+        s->allocs.resize(had);
+        for (const Buffer& b : buffers) *b.ptr = nullptr;
+        return false;
     }
-    s->allocs.push_back({base, body});
-    return b + kGuardBytes;
+    s->blocks.push_back(block);
+    return true;
 }
 
 Couplings couplings(double G1, double G2)
@@ -198,14 +215,26 @@ lb_status fail_cuda(lb_state* s)
     return LB_ERR_CUDA;
 }
 
-// Read the state's control words (synchronises the stream) and the kernels' error flags
-// among them: bit 1, a bounded wait ran out (the state is poisoned); bit 2, a fused
-// reduction produced a non-finite mass or energy (the lattice has blown up).
+// The state's control words into c (synchronises the stream).
+cudaError_t copy_control(lb_state* s, Control& c)
+{
+    char h[kControlBytes];
+    cudaError_t e = cudaMemcpyAsync(h, s->res, sizeof(h), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return e;
+    std::memcpy(c.res, h, sizeof(c.res));
+    std::memcpy(&c.err, h + kControlPitch, sizeof(int));
+    std::memcpy(&c.trace_count, h + 2 * kControlPitch, sizeof(int));
+    std::memcpy(&c.flag, h + 3 * kControlPitch, sizeof(int));
+    return cudaSuccess;
+}
+
+// Read them and the kernels' error flags among them: bit 1, a bounded wait ran out (the
+// state is poisoned); bit 2, a fused reduction produced a non-finite mass or energy (the
+// lattice has blown up).
 lb_status read_control(lb_state* s, Control& c)
 {
-    if (cudaMemcpyAsync(&c, s->res, sizeof(c), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
-        cudaStreamSynchronize(s->stream) != cudaSuccess)
-        return fail_cuda(s);
+    if (copy_control(s, c) != cudaSuccess) return fail_cuda(s);
     if (c.err & 1) {
         s->poisoned = true;
         return LB_ERR_TIMEOUT;
@@ -229,7 +258,7 @@ void free_state(lb_state* s)
     if (!s) return;
     DeviceScope dev(s->p.device);
     cudaStreamSynchronize(s->stream);
-    for (const lb_state::Alloc& a : s->allocs) cudaFree(a.base);
+    for (void* b : s->blocks) cudaFree(b);
     cudaGetLastError();
     delete s;
 }
@@ -398,10 +427,6 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
         delete s;
         return LB_ERR_CUDA;
     }
-    auto alloc = [&](void** q, size_t bytes) -> bool {
-        *q = state_alloc(s, bytes);
-        return *q != nullptr;
-    };
     s->launch = default_launch(p->nx, p->ny, p->prec);
     size_t nblk_step = (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0});
     const size_t nblk_bulk =
@@ -411,33 +436,28 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     // the reduction step's grid sum keeps one total per CTA row after the CTA partials
     s->max_cta_rows = (p->ny + kMinRows - 1) / kMinRows;
     s->partials_cap += (size_t)s->max_cta_rows;
-    bool ok = alloc((void**)&s->partials, 4 * sizeof(double) * s->partials_cap) &&
-              alloc((void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols);
-    Control* ctl = nullptr;
-    ok = ok && alloc((void**)&ctl, sizeof(Control));
-    if (ok) {
-        s->res = ctl->res;
-        s->err = &ctl->err;
-        s->trace_count = &ctl->trace_count;
-        s->flag = &ctl->flag;
-        s->counter = ctl->counter;
-    }
+    // the control words: cleared below, from res to the last counter's guard
+    bool ok = state_alloc(s, {{(void**)&s->res, 4 * sizeof(double)},
+                              {(void**)&s->err, sizeof(int)},
+                              {(void**)&s->trace_count, sizeof(int)},
+                              {(void**)&s->flag, sizeof(int)},
+                              {(void**)&s->counter, 2 * sizeof(unsigned int)}}) &&
+              state_alloc(s, {{(void**)&s->partials, 4 * sizeof(double) * s->partials_cap}}) &&
+              state_alloc(s, {{(void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols}});
     if (ok && p->prec == LB_FP64) {
-        ok = alloc((void**)&s->f64[0], 9 * sizeof(double) * N) &&
-             alloc((void**)&s->f64[1], 9 * sizeof(double) * N) &&
-             alloc((void**)&s->psi64, sizeof(double) * N) &&
-             alloc((void**)&s->rho64, sizeof(double) * N);
+        ok = state_alloc(s, {{(void**)&s->f64[0], 9 * sizeof(double) * N}}) &&
+             state_alloc(s, {{(void**)&s->f64[1], 9 * sizeof(double) * N}}) &&
+             state_alloc(s, {{(void**)&s->psi64, sizeof(double) * N}}) &&
+             state_alloc(s, {{(void**)&s->rho64, sizeof(double) * N}});
     } else if (ok) {
-        const size_t es = elem_size(p->prec);
-        const size_t gb = es * (size_t)g_elems(p->nx, p->ny);
-        const size_t dev_at = ((size_t)N + 63) / 64 * 64;   // aligned as a buffer of its own
-        ok = alloc(&s->g[0], gb) && alloc(&s->g[1], gb) &&
-             alloc((void**)&s->dpsi[0], sizeof(float) * N) &&
-             alloc((void**)&s->dpsi[1], sizeof(float) * (p->trace_every > 0 ? dev_at + N : N));
-        if (p->trace_every > 0) s->dev = s->dpsi[1] + dev_at;
+        const size_t gb = elem_size(p->prec) * (size_t)g_elems(p->nx, p->ny);
+        std::vector<Buffer> psi1 = {{(void**)&s->dpsi[1], sizeof(float) * N}};
+        if (p->trace_every > 0) psi1.push_back({(void**)&s->dev, sizeof(float) * N});
+        ok = state_alloc(s, {{&s->g[0], gb}}) && state_alloc(s, {{&s->g[1], gb}}) &&
+             state_alloc(s, {{(void**)&s->dpsi[0], sizeof(float) * N}}) && state_alloc(s, psi1);
     }
     ResidentBuf& rb = s->res_buf;
-    size_t word_bytes = 0;
+    size_t words4 = 0, words2 = 0;   // bytes of the halo words
     if (ok && alone && p->prec != LB_FP64) {
         int sms = 0;
         const bool om1 = (float)p->omega == 1.0f;
@@ -447,26 +467,21 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
         }
         if (resident_plan(p->nx, p->ny, om1, sms, rb)) {
             rb.trace_every = p->trace_every;
-            word_bytes = resident_words(N, om1);
-            size_t bytes = word_bytes + 256;
-            // partials of one trace row: of the smallest CTAs a shape may have, and CTA rows
-            const size_t row_cap = (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0}) +
-                                   (size_t)s->max_cta_rows;
+            words4 = sizeof(uint4) * 2 * (om1 ? 1 : 3) * (size_t)N;
+            words2 = sizeof(uint2) * 2 * (size_t)N;
+            std::vector<Buffer> held = {{(void**)&rb.llm, words4}, {(void**)&rb.llp, words2}};
             if (p->trace_every > 0) {
                 const long long rows = (8LL << 20) / (8 * N);
                 rb.max_rows = (int)(rows < 2 ? 2 : rows > 16 ? 16 : rows);
-                bytes += (size_t)rb.max_rows * (8 * (size_t)N + 4 * sizeof(double) * row_cap);
+                // partials of one trace row: of the smallest CTAs a shape may have, and CTA rows
+                const size_t row_cap =
+                    (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0}) +
+                    (size_t)s->max_cta_rows;
+                held.push_back({(void**)&rb.counters, sizeof(unsigned int) * (1 + (size_t)rb.max_rows)});
+                held.push_back({(void**)&rb.partials, (size_t)rb.max_rows * 4 * sizeof(double) * row_cap});
+                held.push_back({(void**)&rb.dump, (size_t)rb.max_rows * 2 * sizeof(float) * N});
             }
-            char* m = nullptr;
-            ok = alloc((void**)&m, bytes);
-            if (ok) {
-                // the words and counters first: they start cleared
-                rb.counters = reinterpret_cast<unsigned int*>(m);
-                rb.llm = reinterpret_cast<uint4*>(m + 256);
-                rb.llp = reinterpret_cast<uint2*>(rb.llm + (size_t)2 * (om1 ? 1 : 3) * N);
-                rb.partials = reinterpret_cast<double*>(m + 256 + word_bytes);
-                rb.dump = reinterpret_cast<float*>(rb.partials + (size_t)rb.max_rows * 4 * row_cap);
-            }
+            ok = state_alloc(s, held);
         }
     }
     if (!ok) {
@@ -485,18 +500,17 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     };
     if (cudaMemcpyAsync(rho_in, rho_init, sizeof(double) * N, cudaMemcpyDefault, s->stream) !=
             cudaSuccess ||
-        cudaMemsetAsync(ctl, 0, sizeof(Control), s->stream) != cudaSuccess ||
-        (rb.gx > 0 &&
-         cudaMemsetAsync(rb.counters, 0, 256 + word_bytes, s->stream) != cudaSuccess))
+        cudaMemset2DAsync(s->res, kControlPitch, 0, kGuardBytes, 5, s->stream) != cudaSuccess ||
+        (rb.gx > 0 && (cudaMemsetAsync(rb.llm, 0, words4, s->stream) != cudaSuccess ||
+                       cudaMemsetAsync(rb.llp, 0, words2, s->stream) != cudaSuccess)) ||
+        (rb.counters && cudaMemsetAsync(rb.counters, 0, kGuardBytes, s->stream) != cudaSuccess))
         return bail(LB_ERR_CUDA);
     if (rho_check_sum(rho_in, N, s->partials, s->counter, s->res, s->flag, s->stream) !=
         cudaSuccess)
         return bail(LB_ERR_CUDA);
     Control got{};
     // after this synchronisation the caller's rho_init is no longer read
-    if (cudaMemcpyAsync(&got, ctl, sizeof(got), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
-        cudaStreamSynchronize(s->stream) != cudaSuccess)
-        return bail(LB_ERR_CUDA);
+    if (copy_control(s, got) != cudaSuccess) return bail(LB_ERR_CUDA);
     const double sum = got.res[0];
     if (got.flag) return bail(LB_ERR_ARG);
     // The reference density is rounded to FP32 once: the kernels add it in FP32,

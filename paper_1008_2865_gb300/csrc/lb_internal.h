@@ -235,7 +235,6 @@ struct ResidentBuf {
     unsigned int* counters = nullptr;     // [1 + max_rows]
 };
 bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b);
-size_t resident_words(long long n, bool om1);   // bytes of the halo words
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps,
                           cudaStream_t s);
 cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps,
@@ -286,12 +285,22 @@ cudaError_t fp64_exp_cr(const double* x, double* y, long long n, cudaStream_t s)
 }  // namespace lbsc
 
 namespace lbsc {
-// The words of a state the host reads back, together in one transfer, and the counters.
+constexpr size_t kGuardBytes = 256;              // guard region on each side of a buffer
+constexpr unsigned char kGuardByte = 0xA5;       // the pattern the guards hold
+// The usable size of a guarded buffer: its tail guard starts 256-byte aligned
+constexpr size_t guarded_size(size_t bytes)
+{
+    return (bytes + kGuardBytes - 1) / kGuardBytes * kGuardBytes;
+}
+
+// The control words of a state, each a guarded buffer of its own, in one allocation in this
+// order, so that the host reads back all but the arrival counters in one transfer.
 struct Control {
     double res[4];
     int err, trace_count, flag;
-    unsigned int counter[2];
 };
+constexpr size_t kControlPitch = 3 * kGuardBytes;   // from one word to the next: guards and words
+constexpr size_t kControlBytes = 3 * kControlPitch + sizeof(int);   // res to flag
 }  // namespace lbsc
 
 // The state behind the opaque lb_state* of the C ABI (lb_api.cu owns its
@@ -325,26 +334,37 @@ struct lb_state {
     unsigned int* counter = nullptr;
     double* trace = nullptr;
     int* trace_count = nullptr;
-    double* res = nullptr;         // 4 doubles of results; err and trace_count follow them
+    double* res = nullptr;         // 4 doubles of results; err, trace_count, flag follow (Control)
     int* flag = nullptr;
     double* field_tmp = nullptr;   // N doubles, allocated on the first lb_fields into pageable host memory
-    // every device buffer of the state, with a guard region on each side
+    // every device buffer of the state, with a guard region on each side (base: the first
+    // guard), and the allocations that they lie in
     struct Alloc {
         void* base;
         size_t bytes;
     };
     std::vector<Alloc> allocs;
+    std::vector<void*> blocks;
 };
 
 namespace lbsc {
 // lb_init; `alone`: the state is stepped by itself (false for a batch's replicas)
 lb_status state_init(lb_state** out, const lb_params* p, const double* rho_init, void* stream,
                      bool alone);
-constexpr size_t kGuardBytes = 256;              // guard region on each side of a buffer
-constexpr unsigned char kGuardByte = 0xA5;       // the pattern the guards hold
-// Allocate `bytes` for a state with guards on both sides (pattern written on
-// the state's stream); returns the usable pointer or nullptr.
-void* state_alloc(lb_state* s, size_t bytes);
+// Allocate buffers for a state together, each with guards on both sides (pattern written on
+// the state's stream); the usable pointers are stored in order. False, with nothing allocated,
+// if there is not the memory.
+struct Buffer {
+    void** ptr;
+    size_t bytes;
+};
+bool state_alloc(lb_state* s, const std::vector<Buffer>& buffers);
+// one buffer; nullptr if there is not the memory
+inline void* state_alloc(lb_state* s, size_t bytes)
+{
+    void* p = nullptr;
+    return state_alloc(s, {{&p, bytes}}) ? p : nullptr;
+}
 }  // namespace lbsc
 
 namespace lbsc {

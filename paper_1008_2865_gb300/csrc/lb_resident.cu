@@ -451,8 +451,6 @@ bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b)
     return b.gx > 0;
 }
 
-size_t resident_words(long long n, bool om1) { return (size_t)n * 2 * (sizeof(uint2) + (om1 ? 1 : 3) * sizeof(uint4)); }
-
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
 {
     return resident_steps<float>(a, b, block_x, steps, s);
