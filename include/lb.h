@@ -93,6 +93,10 @@ typedef struct lb_state lb_state;   /* opaque; owns device memory */
  *             FP16 state, stored in 32-column tiles) below 2^31
  *   rho_init  N initial densities, host or device, each finite and > 0
  *   stream    cudaStream_t (as void*) used by every later call on the state
+ * Beside its populations and psi an FP32 or FP16 state takes memory that lets steps share
+ * a launch (lb_step): 4 bytes per site if it has a trace, and for a lattice that fits the
+ * SMs 48 bytes per site (omega = 1; otherwise 112) and, with a trace, 8 bytes per site for
+ * each of 2 to 16 states. Where that cannot be had, the steps are taken without it.
  * Errors: LB_ERR_ARG (bad parameter or rho_init), LB_ERR_OOM, LB_ERR_CUDA. */
 lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, void* stream);
 

@@ -311,10 +311,11 @@ lb_status step_streamed(lb_state* s, long n, bool pairs)
     const bool bulk = s->launch.pipeline == 1;
     pairs = pairs && pairs_pay(s->N);
     // one pair fewer if the buffers would not swap as single steps swap them
-    int singles = pairs && s->in_graphs && pairs_made(s->t, n, te) % 2 != 0 ? 2 : 0;
+    const bool traced = s->dev != nullptr;
+    int singles = pairs && s->in_graphs && pairs_made(s->t, n, te, traced) % 2 != 0 ? 2 : 0;
     while (n > 0) {
         const bool reduce = te > 0 && s->t % te == 0;
-        bool pair = pairs && pair_at(s->t, n, te);
+        bool pair = pairs && pair_at(s->t, n, te, traced);
         if (singles == 1 || (singles == 2 && pair)) {
             --singles;
             pair = false;
@@ -451,11 +452,13 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
              state_alloc(s, {{(void**)&s->rho64, sizeof(double) * N}});
     } else if (ok) {
         const size_t gb = elem_size(p->prec) * (size_t)g_elems(p->nx, p->ny);
-        std::vector<Buffer> psi1 = {{(void**)&s->dpsi[1], sizeof(float) * N}};
-        if (p->trace_every > 0) psi1.push_back({(void**)&s->dev, sizeof(float) * N});
         ok = state_alloc(s, {{&s->g[0], gb}}) && state_alloc(s, {{&s->g[1], gb}}) &&
-             state_alloc(s, {{(void**)&s->dpsi[0], sizeof(float) * N}}) && state_alloc(s, psi1);
+             state_alloc(s, {{(void**)&s->dpsi[0], sizeof(float) * N}}) &&
+             state_alloc(s, {{(void**)&s->dpsi[1], sizeof(float) * N}});
     }
+    // what only faster ways to step need: without the memory for it the state does without
+    if (ok && p->prec != LB_FP64 && p->trace_every > 0)
+        state_alloc(s, {{(void**)&s->dev, sizeof(float) * N}});
     ResidentBuf& rb = s->res_buf;
     size_t words4 = 0, words2 = 0;   // bytes of the halo words
     if (ok && alone && p->prec != LB_FP64) {
@@ -481,7 +484,7 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
                 held.push_back({(void**)&rb.partials, (size_t)rb.max_rows * 4 * sizeof(double) * row_cap});
                 held.push_back({(void**)&rb.dump, (size_t)rb.max_rows * 2 * sizeof(float) * N});
             }
-            ok = state_alloc(s, held);
+            if (!state_alloc(s, held)) rb = ResidentBuf{};
         }
     }
     if (!ok) {

@@ -38,6 +38,7 @@ struct lb_batch {
     int4* d_pair_tiles = nullptr;   // work list of the steps taken two at a time (lb_pair.cu)
     int npair_tiles = 0;
     bool odd = false;               // some replica has an odd nx
+    bool traced_pairs = true;       // every replica can keep a traced state's deviations
     // graphs of one period of steps, starting at t % period == 0 with buffers 0 or 1 in
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -194,7 +195,7 @@ bool build_graph(lb_batch* b, int cur)
     cudaError_t e = cudaSuccess;
     int in = cur;
     for (int k = 0; k < b->period && e == cudaSuccess;) {
-        const bool pair = pair_at(k, b->period - k, b->trace_every);
+        const bool pair = pair_at(k, b->period - k, b->trace_every, b->traced_pairs);
         e = enqueue_steps(b, b->cap, k, in, pair);
         k += pair ? 2 : 1;
         in ^= 1;
@@ -261,6 +262,7 @@ lb_status lb_batch_init(lb_batch** out, int count, const lb_params* params,
         b->om1 = b->om1 && params[r].omega == 1.0;
         b->alternate = b->alternate || marches_alternate(s->N);
         b->odd = b->odd || (s->p.nx & 1);
+        b->traced_pairs = b->traced_pairs && (s->dev || b->trace_every == 0);
     }
     DeviceScope dev(b->device);
     if (!dev.ok ||
@@ -294,7 +296,8 @@ lb_status lb_batch_step(lb_batch* b, long n)
     // from then on as many pairs are taken as swap the buffers alike, without the period's graph
     const bool captures = stream_captures(b->stream);
     b->in_graphs = b->in_graphs || (captures && n > 0);
-    int singles = b->in_graphs && pairs_made(b->t, n, b->trace_every) % 2 != 0 ? 2 : 0;
+    int singles =
+        b->in_graphs && pairs_made(b->t, n, b->trace_every, b->traced_pairs) % 2 != 0 ? 2 : 0;
     while (n > 0) {
         if (b->use_graph && !b->in_graphs && b->period > 0 && b->t % b->period == 0 &&
             n >= b->period && build_graph(b, b->cur)) {
@@ -303,7 +306,7 @@ lb_status lb_batch_step(lb_batch* b, long n)
             n -= b->period;
             b->cur ^= b->period_flips;
         } else {
-            bool pair = !captures && pair_at(b->t, n, b->trace_every);
+            bool pair = !captures && pair_at(b->t, n, b->trace_every, b->traced_pairs);
             if (singles == 1 || (singles == 2 && pair)) {
                 --singles;
                 pair = false;

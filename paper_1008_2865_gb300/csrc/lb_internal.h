@@ -314,7 +314,8 @@ struct lb_state {
     // FP32 / FP16 deviation storage (g tiled, lbsc::g_elems elements each)
     void* g[2] = {nullptr, nullptr};
     float* dpsi[2] = {nullptr, nullptr};
-    float* dev = nullptr;          // density deviations of a traced state (in dpsi[1]'s buffer)
+    float* dev = nullptr;          // density deviations of a traced state; if there was not the
+                                   // memory for them, traced states are stepped singly
     int cur = 0;
     double rho_ref = 0.0;
     lbsc::Fp32Launch launch{128, 64, 0};
@@ -369,20 +370,21 @@ inline void* state_alloc(lb_state* s, size_t bytes)
 
 namespace lbsc {
 // Whether steps t and t + 1 go through a lattice or batch together when `left` steps are
-// left: not when state t + 1 has a trace row (every te steps; 0: none).
-inline bool pair_at(long long t, long long left, int te)
+// left: not when state t + 1 has a trace row (every te steps; 0: none), and when state t has
+// one only if `traced`.
+inline bool pair_at(long long t, long long left, int te, bool traced)
 {
-    return left >= 2 && !(te > 0 && (t + 1) % te == 0);
+    return left >= 2 && !(te > 0 && ((t + 1) % te == 0 || (!traced && t % te == 0)));
 }
 // How many pairs n steps from t make. A captured graph reads and writes the buffers that
 // were in place when it was captured, and its replays are valid after any number of further
 // steps that swaps the buffers as often, modulo two, as single steps do: once each. A pair swaps
 // them once for two steps, so states whose steps have been captured take an even number of pairs.
-inline long long pairs_made(long long t, long long n, int te)
+inline long long pairs_made(long long t, long long n, int te, bool traced)
 {
     long long pairs = 0;
     for (long long k = 0; k < n;) {
-        const bool pair = pair_at(t + k, n - k, te);
+        const bool pair = pair_at(t + k, n - k, te, traced);
         pairs += pair;
         k += pair ? 2 : 1;
     }
