@@ -106,7 +106,8 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
  * then streaming. States t with t % trace_every == 0 append a trace row.
  * Steps may share a launch: an FP32 or FP16 lattice that fits the SMs' shared memory
  * (about 690 x 690 with omega = 1) takes all n in one cooperative launch, others two
- * at a time; the results are those of single steps, bit for bit. In a stream capture
+ * at a time, as does a small one whose stream has fewer SMs than that launch needs; the
+ * results are those of single steps, bit for bit. In a stream capture
  * every step is a launch of its own; a graph of an even number of steps continues the
  * run whenever an even number of steps has been taken outside it since its capture.
  * Asynchronous. Errors: LB_ERR_ARG (n < 0), LB_ERR_STATE, LB_ERR_CUDA. */

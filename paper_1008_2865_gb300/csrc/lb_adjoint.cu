@@ -453,6 +453,7 @@ __global__ void __launch_bounds__(kRevThreads, 1) k_adj_reverse(const RevArgs R)
 {
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_fail, s_nl;
+    if (R.steps == 0) return;                            // asked whether the launch is taken
     const AdjArgs& A = R.A;
     const StepArgs<float>& a = A.a;
     const int tid = threadIdx.x, nt = blockDim.x, warps = nt >> 5, warp = tid >> 5, lane = tid & 31;
@@ -700,6 +701,28 @@ bool reverse_plan(int nx, int ny, int num_sms, RevArgs& R, int& tiles)
     return best < 1e30;
 }
 
+cudaError_t launch_reverse(const RevArgs& R, int tiles, cudaStream_t s)
+{
+    const int sites = (R.tw + 4) * (R.th + 4);
+    int threads = (sites + 31) / 32 * 32;
+    threads = threads < 256 ? 256 : threads > kRevThreads ? kRevThreads : threads;
+    // the limit, not this launch's size: another thread may be launching another lattice
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_adj_reverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeldSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(tiles);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = sizeof(float) * (size_t)rev_floats(R.tw, R.th);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;   // every tile waits for its neighbours'
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_adj_reverse, R);
+}
+
 __global__ void k_adj_grad_init(const float* __restrict__ lam, const float4* __restrict__ lam4, int N,
                                 float w0, float w1, float w2, double* __restrict__ out)
 {
@@ -804,8 +827,20 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
         cudaGetLastError();
         sms = 0;
     }
-    const bool held = (float)s->p.omega == 1.0f && s->res_buf.gx > 0 &&
-                      reverse_plan(s->p.nx, s->p.ny, sms, R, rev_tiles);
+    bool held = (float)s->p.omega == 1.0f && s->res_buf.gx > 0 &&
+                reverse_plan(s->p.nx, s->p.ny, sms, R, rev_tiles);
+    if (held) {
+        // not where the stream refuses either launch, as found out before anything depends on it
+        R.steps = 0;
+        cudaError_t e = fp32_resident_probe(state_args<float>(s, s->cur), s->res_buf, s->stream);
+        if (e == cudaSuccess) e = launch_reverse(R, rev_tiles, s->stream);
+        if (e != cudaSuccess && !launch_refused(e)) {
+            s->poisoned = true;
+            return LB_ERR_CUDA;
+        }
+        held = e == cudaSuccess;
+        cudaGetLastError();
+    }
     const int grid = adj_grid(N);
     const long long rows = T < C ? T : C;                 // steps of a segment at most
     const size_t seg_slots = (size_t)(C > 1 ? C - 1 : 1);
@@ -948,24 +983,6 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
         R.words = words;
         R.states = seg;
         R.terms = terms;
-        const size_t smem = sizeof(float) * (size_t)rev_floats(R.tw, R.th);
-        const int sites = (R.tw + 4) * (R.th + 4);
-        int threads = (sites + 31) / 32 * 32;
-        threads = threads < 256 ? 256 : threads > kRevThreads ? kRevThreads : threads;
-        // the limit, not this launch's size: another thread may be launching another lattice
-        if (cudaFuncSetAttribute(k_adj_reverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kHeldSmem) != cudaSuccess)
-            return fail();
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(rev_tiles);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeCooperative;   // every tile waits for its neighbours'
-        at.val.cooperative = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
         for (long long k = K - 1; k >= 0; --k) {
             const int n = (int)seg_len(k);
             StepArgs<float> a = base;
@@ -978,7 +995,7 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
             R.steps = n;
             R.lam_in = lam4[in4];
             R.lam_out = lam4[in4 ^ 1];
-            if (cudaLaunchKernelEx(&cfg, k_adj_reverse, R) != cudaSuccess || !add_terms(n))
+            if (launch_reverse(R, rev_tiles, st) != cudaSuccess || !add_terms(n))
                 return fail();
             R.tag += (unsigned)n;
             in4 ^= 1;

@@ -264,10 +264,12 @@ void free_state(lb_state* s)
 }
 
 // Steps of a small lattice that stay on the SMs (lb_resident.cu), as many per launch as the
-// trace rows they append can be kept.
-lb_status step_held(lb_state* s, long n)
+// trace rows they append can be kept. `left` receives the steps not taken: none, or all from
+// the launch on that the stream refused.
+lb_status step_held(lb_state* s, long n, long& left)
 {
     ResidentBuf& b = s->res_buf;
+    left = 0;
     while (n > 0) {
         long m = n;
         if (b.trace_every > 0) {
@@ -282,6 +284,12 @@ lb_status step_held(lb_state* s, long n)
             s->p.prec == LB_FP32
                 ? fp32_resident(make_args<float>(s), b, s->launch.block_x, (int)m, s->stream)
                 : fp16_resident(make_args<__half>(s), b, s->launch.block_x, (int)m, s->stream);
+        if (launch_refused(e)) {
+            cudaGetLastError();
+            b.gx = 0;
+            left = n;
+            return LB_OK;
+        }
         if (e != cudaSuccess) return fail_cuda(s);
         s->cur ^= 1;
         s->t += m;
@@ -344,7 +352,10 @@ lb_status step_fp32(lb_state* s, long n)
     const bool captures = stream_captures(s->stream);
     s->in_graphs = s->in_graphs || (captures && n > 0);
     const bool many = n >= 2 && s->launch.pipeline == 0 && !captures;
-    if (many && s->res_buf.gx > 0) return step_held(s, n);
+    if (many && s->res_buf.gx > 0) {
+        const lb_status st = step_held(s, n, n);
+        if (st != LB_OK || n == 0) return st;
+    }
     return step_streamed(s, n, many);
 }
 

@@ -234,6 +234,15 @@ struct ResidentBuf {
     double* partials = nullptr;           // [max_rows][partials of one trace row][4]
     unsigned int* counters = nullptr;     // [1 + max_rows]
 };
+// A cooperative launch is refused, at once and with nothing started, where the stream has fewer
+// SMs than the lattice has tiles (a stream of a green context, a process with a share of
+// the GPU). The steps are then taken without holding the lattice.
+inline bool launch_refused(cudaError_t e)
+{
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
+}
+// Whether the stream takes a held launch of this lattice (a launch without steps).
+cudaError_t fp32_resident_probe(const StepArgs<float>& a, const ResidentBuf& b, cudaStream_t s);
 bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b);
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps,
                           cudaStream_t s);

@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kResThreads<OM1>, 1) k_resident(const ResArgs<
     int* lo = lc + (A.tw + 4) / 2 * (A.th + 2);                   // own pairs
     using TL = Tile<T>;
 
+    if (A.steps == 0) return;                        // asked whether the launch is taken
     if (tid == 0) s_fail = s_np = s_nm = 0;
     __syncthreads();
     // ---- dpsi(t) of the tile and three rings around it; lists of the halo sites
@@ -383,7 +384,6 @@ cudaError_t resident_launch(const StepArgs<T>& a, ResidentBuf& b, int steps, flo
     A.dump = dump;
     A.planes = planes;
     A.keep_every = keep_every;
-    b.tag += (unsigned)steps;
     const bool om1 = a.omega == 1.0f;
     const size_t smem = res_smem(b.tw, b.th, om1);
     // a thread per collision pair and per halo word, from 256 on (us per step, 256 / 384 /
@@ -394,8 +394,10 @@ cudaError_t resident_launch(const StepArgs<T>& a, ResidentBuf& b, int steps, flo
     int threads = ((pairs > words ? pairs : words) + 31) / 32 * 32;
     const int most = om1 ? kResThreads<true> : kResThreads<false>;
     threads = threads < 256 ? 256 : threads > most ? most : threads;
-    return om1 ? launch_resident<T, true>(A, b.gx * b.gy, threads, smem, s)
-               : launch_resident<T, false>(A, b.gx * b.gy, threads, smem, s);
+    const cudaError_t e = om1 ? launch_resident<T, true>(A, b.gx * b.gy, threads, smem, s)
+                              : launch_resident<T, false>(A, b.gx * b.gy, threads, smem, s);
+    if (e == cudaSuccess) b.tag += (unsigned)steps;
+    return e;
 }
 
 template <typename T>
@@ -459,6 +461,11 @@ cudaError_t fp32_resident_kept(const StepArgs<float>& a, ResidentBuf& b, int ste
                                cudaStream_t s)
 {
     return resident_launch<float>(a, b, steps, states, 4, 1, s);
+}
+cudaError_t fp32_resident_probe(const StepArgs<float>& a, const ResidentBuf& b, cudaStream_t s)
+{
+    ResidentBuf none = b;
+    return resident_launch<float>(a, none, 0, nullptr, 2, 0, s);
 }
 cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
 {
