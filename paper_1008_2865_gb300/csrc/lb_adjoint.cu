@@ -145,6 +145,7 @@ struct AdjArgs {
     double* partials;
     unsigned int* counter;
     double* acc;              // [4] FP64 accumulators
+    int* narrow;              // flags of the terminal kernel's sums
 };
 
 // s += x with Kahan's compensation c (the rounding error of the previous adds).
@@ -236,15 +237,18 @@ __device__ void accumulate_grid2(float v0, float v1, const AdjArgs& A)
 // dE/dG1, dE/dG2 (lb_objective takes J alone; its sums are the same additions). T is the
 // population storage type. Rows of CTAs' sites are read as in k_delta_energy; a thread's
 // sums of psi times a class sum are exact FP32 products in two FP32 values (Two), the
-// misfit, whose target is FP64, is summed in FP64.
-template <typename T, bool GRAD>
+// misfit, whose target is FP64, is summed in FP64. A thread whose sums leave the range of Two
+// (as in k_delta_energy) sets bit 1 (E) or 2 (the derivatives) of *A.narrow, and these are
+// taken again with WIDE, in FP64 and without the adjoint.
+template <typename T, bool GRAD, bool WIDE>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_terminal(const AdjArgs A,
                                                               const T* __restrict__ gT)
 {
     const StepArgs<float>& a = A.a;
     const int nx = a.nx, ny = a.ny, N = (int)a.N;
     Two e{0.f, 0.f}, e1{0.f, 0.f}, e2{0.f, 0.f};
-    double mis2 = 0.0;
+    float most = 0.f, most1 = 0.f;            // largest terms of e and e1
+    double mis2 = 0.0, w0 = 0.0, w1 = 0.0, w2 = 0.0;
     for (int s = blockIdx.x * kAdjThreads + threadIdx.x; s < N; s += gridDim.x * kAdjThreads) {
         const int y = s / nx, x = s - y * nx;
         const double target = __ldg(A.rho_target + s);
@@ -267,16 +271,25 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_terminal(const AdjArgs A,
         const float S8 = fmaf(4.f, pr, (p[4][4] + p[4][0]) + (p[0][4] + p[0][0]));
         const float dEdpsi = a.K0 * pc + a.K1 * S1 + a.K2 * S2 + a.K4 * S4 + a.K5 * S5 + a.K8 * S8;
         const double mis = (double)rho - target;
+        mis2 += mis * mis;
+        const float sw = A.aw.K0 * pc + A.aw.K1 * S1 + A.aw.K2 * S2;
+        const float sp = A.ap.K0 * pc + A.ap.K1 * S1 + A.ap.K2 * S2 + A.ap.K4 * S4 +
+                         A.ap.K5 * S5 + A.ap.K8 * S8;
+        if (WIDE) {
+            w0 += 0.5 * (double)pc * dEdpsi;
+            if (GRAD) {
+                w1 += 0.5 * (double)pc * sw;
+                w2 += 0.5 * (double)pc * sp;
+            }
+            continue;
+        }
         auto add_product = [&](Two& sum, float u, float v) {
             const float q = __fmul_rn(u, v);
             two_add(sum, q, __fmaf_rn(u, v, -q));
+            return fabsf(q);
         };
-        add_product(e, pc, dEdpsi);
-        mis2 += mis * mis;
+        most = fmaxf(most, add_product(e, pc, dEdpsi));
         if (GRAD) {
-            const float sw = A.aw.K0 * pc + A.aw.K1 * S1 + A.aw.K2 * S2;
-            const float sp = A.ap.K0 * pc + A.ap.K1 * S1 + A.ap.K2 * S2 + A.ap.K4 * S4 +
-                             A.ap.K5 * S5 + A.ap.K8 * S8;
             const float dpr = __expf(-rho * a.inv_rho0) * A.inv_sqrt_rho0;
             const float lam = dpr * dEdpsi + (float)(2.0 * mis);
             if (A.lam4) {
@@ -285,12 +298,22 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_terminal(const AdjArgs A,
 #pragma unroll
                 for (int i = 0; i < 9; ++i) A.lam[i * N + s] = lam;
             }
-            add_product(e1, pc, sw);
+            most1 = fmaxf(most1, add_product(e1, pc, sw));
             add_product(e2, pc, sp);
         }
     }
+    if (!WIDE) {
+        w0 = 0.5 * value(e);
+        w1 = 0.5 * value(e1);
+        w2 = 0.5 * value(e2);
+        // without couplings E is zero, whatever psi is
+        const bool coupled = a.K0 != 0.f || a.K1 != 0.f || a.K2 != 0.f || a.K4 != 0.f;
+        int bits = (most >= kNarrowLeast || !coupled) && isfinite(w0) ? 0 : 1;
+        if (GRAD && !(most1 >= kNarrowLeast && isfinite(w1) && isfinite(w2))) bits |= 2;
+        if (bits && blockIdx.x * kAdjThreads + threadIdx.x < N) atomicOr(A.narrow, bits);
+    }
     // E, misfit, dE/dG1, dE/dG2
-    double v[4] = {0.5 * value(e), mis2, 0.5 * value(e1), 0.5 * value(e2)};
+    double v[4] = {w0, mis2, w1, w2};
     accumulate_grid<kAdjThreads>(v, A);
 }
 
@@ -929,7 +952,9 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
     float4* lam4[2] = {reinterpret_cast<float4*>(lam), reinterpret_cast<float4*>(lam) + N};
     A.lam4 = held ? lam4[0] : nullptr;
     A.acc = acc;             // acc[0..3] = E, misfit, dE/dG1, dE/dG2
-    k_adj_terminal<float, true><<<grid, kAdjThreads, 0, st>>>(A, A.g);
+    A.narrow = s->flag;
+    const AdjArgs terminal = A;
+    k_adj_terminal<float, true, false><<<grid, kAdjThreads, 0, st>>>(A, A.g);
     if (cudaGetLastError() != cudaSuccess) return fail();
 
     // ---- reverse over the segments. Segment k (states kC .. kC + n - 1) is
@@ -1029,15 +1054,33 @@ extern "C" lb_status lb_adjoint(lb_state* s, long steps, const double* rho_targe
         lamA, held ? lam4[in4] : nullptr, N, A.a.w0, A.a.w1, A.a.w2, gout);
     if (cudaGetLastError() != cudaSuccess) return fail();
     double h[8];
-    int flags = 0;
+    int flags = 0, narrow = 0;
     if (cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&flags, s->err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        cudaMemcpyAsync(&flags, s->err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&narrow, s->flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return fail();
     if (!grad_on_dev &&
         cudaMemcpyAsync(grad_rho, grad_dev, sizeof(double) * N, cudaMemcpyDeviceToHost, st) !=
             cudaSuccess)
         return fail();
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail();
+    if (narrow && !(flags & 1)) {
+        // J or the explicit derivatives beyond the range of the FP32 pairs
+        double w[4];
+        if (cudaMemsetAsync(s->flag, 0, sizeof(int), st) != cudaSuccess ||
+            cudaMemsetAsync(acc, 0, sizeof(w), st) != cudaSuccess)
+            return fail();
+        k_adj_terminal<float, true, true><<<grid, kAdjThreads, 0, st>>>(terminal, terminal.g);
+        if (cudaGetLastError() != cudaSuccess ||
+            cudaMemcpyAsync(w, acc, sizeof(w), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            return fail();
+        if (narrow & 1) h[0] = w[0];
+        if (narrow & 2) {
+            h[2] = w[2];
+            h[3] = w[3];
+        }
+    }
     release();
     if (flags & 1) {                                 // a bounded wait ran out
         s->poisoned = true;
@@ -1070,7 +1113,8 @@ __global__ void __launch_bounds__(256) k_misfit64(const double* __restrict__ rho
 
 namespace lbsc {
 
-cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, cudaStream_t st)
+cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, bool wide,
+                            cudaStream_t st)
 {
     AdjArgs A{};
     A.a = state_args<float>(s, s->cur);
@@ -1084,13 +1128,17 @@ cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, c
     A.partials = s->partials;
     A.counter = s->counter;
     A.acc = acc;
+    A.narrow = s->flag;
     cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const int grid = adj_grid(s->N);
+    auto go = [&](auto kern, auto* g) { kern<<<grid, kAdjThreads, 0, st>>>(A, g); };
+    const auto *f = static_cast<const float*>(s->g[s->cur]);
+    const auto *h = static_cast<const __half*>(s->g[s->cur]);
     if (s->p.prec == LB_FP16_DELTA)
-        k_adj_terminal<__half, false><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const __half*>(s->g[s->cur]));
+        wide ? go(k_adj_terminal<__half, false, true>, h) : go(k_adj_terminal<__half, false, false>, h);
     else
-        k_adj_terminal<float, false><<<grid, kAdjThreads, 0, st>>>(A, static_cast<const float*>(s->g[s->cur]));
+        wide ? go(k_adj_terminal<float, false, true>, f) : go(k_adj_terminal<float, false, false>, f);
     return cudaGetLastError();
 }
 

@@ -575,22 +575,31 @@ lb_status lb_energy(lb_state* s, double out[4])
     if (s->poisoned) return LB_ERR_STATE;
     DeviceScope dev(s->p.device);
     if (!dev.ok) return fail_cuda(s);
-    if (s->p.prec == LB_FP64) {
-        const Fp64Args a = make64(s);
-        LB_CUDA(s, fp64_psi(a, s->stream));
-        LB_CUDA(s, fp64_energy(a, s->partials, s->counter, s->res, nullptr, nullptr, s->t,
-                               s->stream));
-    } else if (s->p.prec == LB_FP32) {
-        const StepArgs<float> a = make_args<float>(s);
-        LB_CUDA(s, delta_energy<float>(a.g_in, a.dpsi_in, s->p.nx, s->p.ny, a, s->res,
-                                       s->partials, s->counter, s->stream));
-    } else {
+    auto sums = [&](bool wide) -> cudaError_t {
+        if (s->p.prec == LB_FP64) {
+            const Fp64Args a = make64(s);
+            const cudaError_t e = fp64_psi(a, s->stream);
+            return e != cudaSuccess ? e
+                                    : fp64_energy(a, s->partials, s->counter, s->res, nullptr, nullptr,
+                                                  s->t, s->stream);
+        }
+        if (s->p.prec == LB_FP32) {
+            const StepArgs<float> a = make_args<float>(s);
+            return delta_energy<float>(a.g_in, a.dpsi_in, s->p.nx, s->p.ny, a, s->res, s->partials,
+                                       s->counter, s->flag, wide, s->stream);
+        }
         const StepArgs<__half> a = make_args<__half>(s);
-        LB_CUDA(s, delta_energy<__half>(a.g_in, a.dpsi_in, s->p.nx, s->p.ny, a, s->res,
-                                        s->partials, s->counter, s->stream));
-    }
+        return delta_energy<__half>(a.g_in, a.dpsi_in, s->p.nx, s->p.ny, a, s->res, s->partials,
+                                    s->counter, s->flag, wide, s->stream);
+    };
+    LB_CUDA(s, sums(false));
     Control c;
-    const lb_status st = read_control(s, c);
+    lb_status st = read_control(s, c);
+    if (st != LB_ERR_CUDA && c.flag) {   // beyond the range of the FP32 pairs
+        LB_CUDA(s, cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream));
+        LB_CUDA(s, sums(true));
+        st = read_control(s, c);
+    }
     if (st != LB_OK) return st;
     for (int k = 0; k < 4; ++k) out[k] = c.res[k];
     for (int k = 0; k < 4; ++k)
@@ -630,10 +639,15 @@ lb_status lb_objective(lb_state* s, const double* rho_target, double* J)
         LB_CUDA(s, misfit64(s->rho64, tgt, N, s->partials, s->counter, s->res, s->stream));
     } else {
         // the terminal sums of lb_adjoint (same kernel, grid and order)
-        LB_CUDA(s, objective_delta(s, tgt, s->res, s->stream));
+        LB_CUDA(s, objective_delta(s, tgt, s->res, false, s->stream));
     }
     Control c;
-    const lb_status st = read_control(s, c);
+    lb_status st = read_control(s, c);
+    if (st != LB_ERR_CUDA && c.flag) {   // beyond the range of the FP32 pairs
+        LB_CUDA(s, cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream));
+        LB_CUDA(s, objective_delta(s, tgt, s->res, true, s->stream));
+        st = read_control(s, c);
+    }
     if (st == LB_ERR_CUDA) return st;
     *J = s->p.prec == LB_FP64 ? (h[0] + h[1]) + c.res[0] : c.res[0] + c.res[1];
     return st != LB_OK || std::isfinite(*J) ? st : LB_ERR_NONFINITE;

@@ -366,6 +366,9 @@ __device__ __forceinline__ void two_fma(Two& s, Two a, Two b)
     const float e = __fmaf_rn(a.hi, b.hi, -p);
     two_add(s, p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e)));
 }
+// The least sum of magnitudes that such a sum is trusted with: the rounding errors it keeps
+// are then at least 2^-24 of values that are far from FP32's denormals (2^-126).
+constexpr float kNarrowLeast = 0x1p-80f;
 __device__ __forceinline__ double value(Two s) { return (double)s.hi + (double)s.lo; }
 
 // Deterministic sum of 4 doubles over a CTA of NT threads (NT a multiple of

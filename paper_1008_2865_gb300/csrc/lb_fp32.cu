@@ -472,10 +472,12 @@ __global__ void __launch_bounds__(256) k_delta_fields(const T* __restrict__ g, i
 }
 
 // The couplings of k_delta_energy, formed in FP64 on the host: E_s and E_m of a site are
-// psi/2 times cs + sum K S and cm + sum K S over the class sums S of the deviations.
+// psi/2 times cs + sum K S and cm + sum K S over the class sums S of the deviations. Those
+// of a belt are divided by its unit, a power of two that leaves the largest in 1/2 .. 1.
 struct EnergyArgs {
     Two K0, K1, K2, K4, K5, K8;
     Two cs, cm;      // psi_ref (4 K1 + 4 K2), psi_ref (4 K4 + 8 K5 + 4 K8)
+    double unit1, unit2;
 };
 
 // lb_energy: the Sec. 5 sums and the mass of state t. Row by row (blockIdx.y
@@ -488,14 +490,18 @@ struct EnergyArgs {
 // thread in FP64. (4096^2, the whole call: 827 us with those in FP64, which then bounds the
 // kernel, 25 operations a site at two per clock and SM, 250 us now; the energies differ
 // by less than 1e-15 of their magnitude.)
-template <typename T>
+// FP32 has not the range of FP64: a thread whose sums overflow or meet an infinity, or whose
+// psi^2 sum up to less than 2^-80, so that the low parts lose bits to denormals, sets *narrow,
+// and the call takes the sums again with WIDE, in FP64.
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) k_delta_energy(const T* __restrict__ g,
                                                       const float* __restrict__ dpsi,
                                                       const StepArgs<T> a, const EnergyArgs k,
-                                                      double* out4)
+                                                      double* out4, int* narrow)
 {
     const int nx = a.nx, ny = a.ny;
     Two es{0.f, 0.f}, em{0.f, 0.f}, eb{0.f, 0.f}, ms{0.f, 0.f};
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
         const float* rw[5];
 #pragma unroll
@@ -524,6 +530,18 @@ __global__ void __launch_bounds__(256) k_delta_energy(const T* __restrict__ g,
             const float S5 = ((q[3][4] + q[3][0]) + (q[1][4] + q[1][0])) +
                              ((q[4][3] + q[4][1]) + (q[0][3] + q[0][1]));
             const float S8 = (q[4][4] + q[4][0]) + (q[0][4] + q[0][0]);
+            const float d =
+                ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+            if (WIDE) {
+                const double pr = a.psi_ref, pc = pr + (double)q[2][2];
+                const double b1 = a.K0 * pc + a.K1 * (4 * pr + S1) + a.K2 * (4 * pr + S2);
+                const double b2 = a.K4 * (4 * pr + S4) + a.K5 * (8 * pr + S5) + a.K8 * (4 * pr + S8);
+                v[0] += 0.5 * pc * b1;
+                v[1] += 0.5 * pc * b2;
+                v[2] += (double)a.half_A1 * pc * pc;
+                v[3] += (double)d;
+                continue;
+            }
             Two pc{a.psi_ref, 0.f};
             two_add(pc, q[2][2], 0.f);
             Two b1 = k.cs, b2 = k.cm;
@@ -536,12 +554,19 @@ __global__ void __launch_bounds__(256) k_delta_energy(const T* __restrict__ g,
             two_fma(es, pc, b1);
             two_fma(em, pc, b2);
             two_fma(eb, pc, pc);
-            const float d =
-                ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
             two_add(ms, d, 0.f);
         }
     }
-    double v[4] = {0.5 * value(es), 0.5 * value(em), (double)a.half_A1 * value(eb), value(ms)};
+    if (!WIDE) {
+        v[0] = 0.5 * k.unit1 * value(es);
+        v[1] = 0.5 * k.unit2 * value(em);
+        v[2] = (double)a.half_A1 * value(eb);
+        v[3] = value(ms);
+        const bool any = (int)blockIdx.y < ny && (int)(blockIdx.x * 256 + threadIdx.x) < nx;
+        if (any && !(eb.hi >= kNarrowLeast && isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) &&
+                     isfinite(v[3])))
+            *narrow = 1;
+    }
     if (last_block_total<256>(v, a.partials, a.counter, gridDim.x * gridDim.y)) {
         out4[0] = v[0];
         out4[1] = v[1];
@@ -725,7 +750,8 @@ cudaError_t delta_fields(const T* g, int nx, int ny, double rho_ref, double* rho
 
 template <typename T>
 cudaError_t delta_energy(const T* g, const float* dpsi, int nx, int ny, const StepArgs<T>& a,
-                         double* out4, double* partials, unsigned int* counter, cudaStream_t s)
+                         double* out4, double* partials, unsigned int* counter, int* narrow,
+                         bool wide, cudaStream_t s)
 {
     StepArgs<T> b = a;
     b.partials = partials;
@@ -740,11 +766,20 @@ cudaError_t delta_energy(const T* g, const float* dpsi, int nx, int ny, const St
         const float h = (float)v;
         return Two{h, (float)(v - (double)h)};
     };
-    const double pr = a.psi_ref, K1 = a.K1, K2 = a.K2, K4 = a.K4, K5 = a.K5, K8 = a.K8;
-    const EnergyArgs k{host_two(a.K0), host_two(K1), host_two(K2), host_two(K4), host_two(K5),
+    auto unit_of = [](double k0, double k1, double k2) {
+        const double most = std::fmax(std::fabs(k0), std::fmax(std::fabs(k1), std::fabs(k2)));
+        int e = 0;
+        if (std::isfinite(most) && most > 0.0) std::frexp(most, &e);
+        return std::ldexp(1.0, e);
+    };
+    const double u1 = unit_of(a.K0, a.K1, a.K2), u2 = unit_of(a.K4, a.K5, a.K8);
+    const double pr = a.psi_ref, K0 = a.K0 / u1, K1 = a.K1 / u1, K2 = a.K2 / u1, K4 = a.K4 / u2,
+                 K5 = a.K5 / u2, K8 = a.K8 / u2;
+    const EnergyArgs k{host_two(K0), host_two(K1), host_two(K2), host_two(K4), host_two(K5),
                        host_two(K8), host_two(pr * (4 * K1 + 4 * K2)),
-                       host_two(pr * (4 * K4 + 8 * K5 + 4 * K8))};
-    k_delta_energy<T><<<dim3(bx, by), 256, 0, s>>>(g, dpsi, b, k, out4);
+                       host_two(pr * (4 * K4 + 8 * K5 + 4 * K8)), u1, u2};
+    if (wide) k_delta_energy<T, true><<<dim3(bx, by), 256, 0, s>>>(g, dpsi, b, k, out4, narrow);
+    else k_delta_energy<T, false><<<dim3(bx, by), 256, 0, s>>>(g, dpsi, b, k, out4, narrow);
     return cudaGetLastError();
 }
 
@@ -765,9 +800,9 @@ template cudaError_t delta_fields<__half>(const __half*, int, int, double, doubl
                                           double*, cudaStream_t);
 template cudaError_t delta_energy<float>(const float*, const float*, int, int,
                                          const StepArgs<float>&, double*, double*, unsigned int*,
-                                         cudaStream_t);
+                                         int*, bool, cudaStream_t);
 template cudaError_t delta_energy<__half>(const __half*, const float*, int, int,
                                           const StepArgs<__half>&, double*, double*,
-                                          unsigned int*, cudaStream_t);
+                                          unsigned int*, int*, bool, cudaStream_t);
 
 }  // namespace lbsc

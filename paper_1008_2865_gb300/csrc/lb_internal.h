@@ -265,7 +265,8 @@ cudaError_t delta_fields(const T* g, int nx, int ny, double rho_ref, double* rho
                          double* uy, cudaStream_t s);
 template <typename T>
 cudaError_t delta_energy(const T* g, const float* dpsi, int nx, int ny, const StepArgs<T>& a,
-                         double* out4, double* partials, unsigned int* counter, cudaStream_t s);
+                         double* out4, double* partials, unsigned int* counter, int* narrow,
+                         bool wide, cudaStream_t s);
 
 // Input checks and sums (lb_fp32.cu): out[0] = sum rho, flag |= 1 if any rho is
 // not finite or <= 0.
@@ -409,8 +410,10 @@ size_t elem_size(lb_precision p);
 double* device_view(double* p);
 // Objective sums of lb_adjoint's terminal kernel for an FP32/FP16 state
 // (lb_adjoint.cu): acc[0] = E_s + E_m of the current state, acc[1] = sum (rho -
-// tgt)^2, acc[2..3] the explicit dE/dG1, dE/dG2; tgt is device memory.
-cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, cudaStream_t st);
+// tgt)^2, acc[2..3] the explicit dE/dG1, dE/dG2; tgt is device memory. wide: in FP64
+// throughout, for states that set the state's flag without it (delta_energy's `narrow`).
+cudaError_t objective_delta(const lb_state* s, const double* tgt, double* acc, bool wide,
+                            cudaStream_t st);
 // *out = sum (rho - tgt)^2 over n doubles in device memory, deterministic.
 cudaError_t misfit64(const double* rho, const double* tgt, long long n, double* partials,
                      unsigned int* counter, double* out, cudaStream_t st);
