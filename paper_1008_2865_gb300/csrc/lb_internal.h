@@ -241,8 +241,9 @@ inline bool launch_refused(cudaError_t e)
 {
     return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
 }
-// Whether the stream takes a held launch of this lattice (a launch without steps).
-cudaError_t fp32_resident_probe(const StepArgs<float>& a, const ResidentBuf& b, cudaStream_t s);
+// Whether the stream takes a held launch of this lattice: one step into the idle buffers. (A
+// test for a launch without steps in the kernel costs 1% of every step at 70x45.)
+cudaError_t fp32_resident_probe(const StepArgs<float>& a, ResidentBuf& b, cudaStream_t s);
 bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b);
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps,
                           cudaStream_t s);

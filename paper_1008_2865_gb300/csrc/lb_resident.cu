@@ -111,7 +111,6 @@ __global__ void __launch_bounds__(kResThreads<OM1>, 1) k_resident(const ResArgs<
     int* lo = lc + (A.tw + 4) / 2 * (A.th + 2);                   // own pairs
     using TL = Tile<T>;
 
-    if (A.steps == 0) return;                        // asked whether the launch is taken
     if (tid == 0) s_fail = s_np = s_nm = 0;
     __syncthreads();
     // ---- dpsi(t) of the tile and three rings around it; lists of the halo sites
@@ -462,10 +461,9 @@ cudaError_t fp32_resident_kept(const StepArgs<float>& a, ResidentBuf& b, int ste
 {
     return resident_launch<float>(a, b, steps, states, 4, 1, s);
 }
-cudaError_t fp32_resident_probe(const StepArgs<float>& a, const ResidentBuf& b, cudaStream_t s)
+cudaError_t fp32_resident_probe(const StepArgs<float>& a, ResidentBuf& b, cudaStream_t s)
 {
-    ResidentBuf none = b;
-    return resident_launch<float>(a, none, 0, nullptr, 2, 0, s);
+    return resident_launch<float>(a, b, 1, nullptr, 2, 0, s);
 }
 cudaError_t fp16_resident(const StepArgs<__half>& a, ResidentBuf& b, int block_x, int steps, cudaStream_t s)
 {
