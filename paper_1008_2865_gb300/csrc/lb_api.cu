@@ -17,20 +17,32 @@ namespace lbsc {
 // Test hook: allocations left before one is made to fail (-1: never).
 static std::atomic<int> g_fail_allocs_after{-1};
 
-bool state_alloc(lb_state* s, const std::vector<Buffer>& buffers)
+bool state_alloc(lb_state* s, std::vector<Buffer> buffers, bool spare_last)
 {
-    size_t total = 0;
-    for (const Buffer& b : buffers) {
+    size_t total = 0, last = 0;
+    auto leave_out_last = [&]() {
+        *buffers.back().ptr = nullptr;
+        buffers.pop_back();
+        spare_last = false;
+    };
+    for (size_t k = 0; k < buffers.size(); ++k) {
         int left = g_fail_allocs_after.load();
         while (left >= 0 && !g_fail_allocs_after.compare_exchange_weak(left, left - 1)) {
         }
-        if (left == 0) return false;   // the hook's failure (counter is now -1: disarmed)
-        total += guarded_size(b.bytes) + 2 * kGuardBytes;
+        if (left == 0) {   // the hook's failure (counter is now -1: disarmed)
+            if (!spare_last || k + 1 < buffers.size()) return false;
+            leave_out_last();
+            break;
+        }
+        last = guarded_size(buffers[k].bytes) + 2 * kGuardBytes;
+        total += last;
     }
     void* block = nullptr;
-    if (cudaMalloc(&block, total) != cudaSuccess) {
+    while (cudaMalloc(&block, total) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        if (!spare_last) return false;
+        leave_out_last();
+        total -= last;
     }
     // the guards: one fill over small buffers and all, otherwise one at each end and where
     // two buffers meet
@@ -448,28 +460,29 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     // the reduction step's grid sum keeps one total per CTA row after the CTA partials
     s->max_cta_rows = (p->ny + kMinRows - 1) / kMinRows;
     s->partials_cap += (size_t)s->max_cta_rows;
-    // the control words: cleared below, from res to the last counter's guard
+    // the control words first, at the distances that kControlPitch states; cleared below
     bool ok = state_alloc(s, {{(void**)&s->res, 4 * sizeof(double)},
                               {(void**)&s->err, sizeof(int)},
                               {(void**)&s->trace_count, sizeof(int)},
                               {(void**)&s->flag, sizeof(int)},
-                              {(void**)&s->counter, 2 * sizeof(unsigned int)}}) &&
-              state_alloc(s, {{(void**)&s->partials, 4 * sizeof(double) * s->partials_cap}}) &&
-              state_alloc(s, {{(void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols}});
+                              {(void**)&s->counter, 2 * sizeof(unsigned int)},
+                              {(void**)&s->partials, 4 * sizeof(double) * s->partials_cap},
+                              {(void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols}});
     if (ok && p->prec == LB_FP64) {
-        ok = state_alloc(s, {{(void**)&s->f64[0], 9 * sizeof(double) * N}}) &&
-             state_alloc(s, {{(void**)&s->f64[1], 9 * sizeof(double) * N}}) &&
-             state_alloc(s, {{(void**)&s->psi64, sizeof(double) * N}}) &&
-             state_alloc(s, {{(void**)&s->rho64, sizeof(double) * N}});
+        ok = state_alloc(s, {{(void**)&s->f64[0], 9 * sizeof(double) * N},
+                             {(void**)&s->f64[1], 9 * sizeof(double) * N},
+                             {(void**)&s->psi64, sizeof(double) * N},
+                             {(void**)&s->rho64, sizeof(double) * N}});
     } else if (ok) {
         const size_t gb = elem_size(p->prec) * (size_t)g_elems(p->nx, p->ny);
-        ok = state_alloc(s, {{&s->g[0], gb}}) && state_alloc(s, {{&s->g[1], gb}}) &&
-             state_alloc(s, {{(void**)&s->dpsi[0], sizeof(float) * N}}) &&
-             state_alloc(s, {{(void**)&s->dpsi[1], sizeof(float) * N}});
+        const bool traced = p->trace_every > 0;
+        std::vector<Buffer> fields = {{&s->g[0], gb},
+                                      {&s->g[1], gb},
+                                      {(void**)&s->dpsi[0], sizeof(float) * N},
+                                      {(void**)&s->dpsi[1], sizeof(float) * N}};
+        if (traced) fields.push_back({(void**)&s->dev, sizeof(float) * N});
+        ok = state_alloc(s, fields, traced);
     }
-    // what only faster ways to step need: without the memory for it the state does without
-    if (ok && p->prec != LB_FP64 && p->trace_every > 0)
-        state_alloc(s, {{(void**)&s->dev, sizeof(float) * N}});
     ResidentBuf& rb = s->res_buf;
     size_t words4 = 0, words2 = 0;   // bytes of the halo words
     if (ok && alone && p->prec != LB_FP64) {
