@@ -138,7 +138,7 @@ Fp32Launch default_launch(int nx, int ny, lb_precision prec)
 {
     (void)prec;
     Fp32Launch L{128, 64, 0};
-    if ((long long)nx * ny * 80 <= (128LL << 20)) L.block_x = 64;
+    if (!beyond_l2((long long)nx * ny)) L.block_x = 64;
     const long long strips = (nx + L.block_x - 3) / (L.block_x - 2);
     const long long target = 152LL * (40 * 32 / L.block_x) * 5;
     long long rows = (strips * ny + target - 1) / target;
@@ -276,13 +276,13 @@ void free_state(lb_state* s)
 }
 
 // Steps of a small lattice that stay on the SMs (lb_resident.cu), as many per launch as the
-// trace rows they append can be kept. `left` receives the steps not taken: none, or all from
-// the launch on that the stream refused.
+// trace rows they append can be kept. `left` receives the steps not taken: too few for a
+// launch at the end, or all from the launch on that the stream refused.
 lb_status step_held(lb_state* s, long n, long& left)
 {
     ResidentBuf& b = s->res_buf;
-    left = 0;
-    while (n > 0) {
+    const int least = held_least(b.tw * b.th, (float)s->p.omega == 1.0f);
+    while (left = n, n >= least) {
         long m = n;
         if (b.trace_every > 0) {
             const long long te = b.trace_every;
@@ -292,6 +292,7 @@ lb_status step_held(lb_state* s, long n, long& left)
         }
         if (m > (1L << 20)) m = 1L << 20;
         if (s->in_graphs && m % 2 == 0) --m;   // a launch swaps the buffers once
+        if (m < least) return LB_OK;
         const cudaError_t e =
             s->p.prec == LB_FP32
                 ? fp32_resident(make_args<float>(s), b, s->launch.block_x, (int)m, s->stream)
@@ -299,7 +300,6 @@ lb_status step_held(lb_state* s, long n, long& left)
         if (launch_refused(e)) {
             cudaGetLastError();
             b.gx = 0;
-            left = n;
             return LB_OK;
         }
         if (e != cudaSuccess) return fail_cuda(s);
@@ -329,9 +329,9 @@ lb_status step_streamed(lb_state* s, long n, bool pairs)
 {
     const int te = s->p.trace_every;
     const bool bulk = s->launch.pipeline == 1;
-    pairs = pairs && pairs_pay(s->N);
+    pairs = pairs && pairs_pay(s->p.nx, s->p.ny, s->launch.block_x);
     // one pair fewer if the buffers would not swap as single steps swap them
-    const bool traced = s->dev != nullptr;
+    const bool traced = s->dev && traced_pairs_pay(s->p.nx, s->p.ny, s->launch.block_x);
     int singles = pairs && s->in_graphs && pairs_made(s->t, n, te, traced) % 2 != 0 ? 2 : 0;
     while (n > 0) {
         const bool reduce = te > 0 && s->t % te == 0;
@@ -499,7 +499,8 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
             std::vector<Buffer> held = {{(void**)&rb.llm, words4}, {(void**)&rb.llp, words2}};
             if (p->trace_every > 0) {
                 const long long rows = (8LL << 20) / (8 * N);
-                rb.max_rows = (int)(rows < 2 ? 2 : rows > 16 ? 16 : rows);
+                const int least = held_least(rb.tw * rb.th, om1) + 1;   // a launch at every state traced
+                rb.max_rows = (int)(rows < least ? least : rows > 16 ? 16 : rows);
                 // partials of one trace row: of the smallest CTAs a shape may have, and CTA rows
                 const size_t row_cap =
                     (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0}) +

@@ -38,7 +38,8 @@ struct lb_batch {
     int4* d_pair_tiles = nullptr;   // work list of the steps taken two at a time (lb_pair.cu)
     int npair_tiles = 0;
     bool odd = false;               // some replica has an odd nx
-    bool traced_pairs = true;       // every replica can keep a traced state's deviations
+    bool pairs = true;              // steps are taken two at a time
+    bool traced_pairs = true;       // also those of a traced state
     // graphs of one period of steps, starting at t % period == 0 with buffers 0 or 1 in
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -117,7 +118,19 @@ lb_status build_tables(lb_batch* b)
     b->ntiles = (int)tiles.size();
     b->nrows = nrows_total;
     std::vector<std::pair<int, int>> sizes;
-    for (const lb_state* s : b->reps) sizes.emplace_back(s->p.nx, s->p.ny);
+    int tallest = 0;
+    long long sites = 0, pair = 0, single = 0;
+    bool kept = true;                   // every replica can keep a traced state's deviations
+    for (const lb_state* s : b->reps) {
+        sizes.emplace_back(s->p.nx, s->p.ny);
+        tallest = std::max(tallest, s->p.ny);
+        kept = kept && s->dev;
+        sites += s->N;
+        pair += pair_columns(s->p.nx) * s->p.ny;
+        single += single_columns(s->p.nx, b->block_x) * s->p.ny;
+    }
+    b->pairs = batch_pairs_pay(sites, pair, single);
+    b->traced_pairs = kept && batch_traced_pairs_pay(tallest, b->rows, (int)elem_size(b->prec));
     std::vector<int4> pair_list;
     pair_tiles(sizes, (int)elem_size(b->prec), b->om1, b->num_sms, pair_list);
     b->npair_tiles = (int)pair_list.size();
@@ -195,7 +208,7 @@ bool build_graph(lb_batch* b, int cur)
     cudaError_t e = cudaSuccess;
     int in = cur;
     for (int k = 0; k < b->period && e == cudaSuccess;) {
-        const bool pair = pair_at(k, b->period - k, b->trace_every, b->traced_pairs);
+        const bool pair = b->pairs && pair_at(k, b->period - k, b->trace_every, b->traced_pairs);
         e = enqueue_steps(b, b->cap, k, in, pair);
         k += pair ? 2 : 1;
         in ^= 1;
@@ -262,7 +275,6 @@ lb_status lb_batch_init(lb_batch** out, int count, const lb_params* params,
         b->om1 = b->om1 && params[r].omega == 1.0;
         b->alternate = b->alternate || marches_alternate(s->N);
         b->odd = b->odd || (s->p.nx & 1);
-        b->traced_pairs = b->traced_pairs && (s->dev || b->trace_every == 0);
     }
     DeviceScope dev(b->device);
     if (!dev.ok ||
@@ -297,7 +309,7 @@ lb_status lb_batch_step(lb_batch* b, long n)
     const bool captures = stream_captures(b->stream);
     b->in_graphs = b->in_graphs || (captures && n > 0);
     int singles =
-        b->in_graphs && pairs_made(b->t, n, b->trace_every, b->traced_pairs) % 2 != 0 ? 2 : 0;
+        b->pairs && b->in_graphs && pairs_made(b->t, n, b->trace_every, b->traced_pairs) % 2 != 0 ? 2 : 0;
     while (n > 0) {
         if (b->use_graph && !b->in_graphs && b->period > 0 && b->t % b->period == 0 &&
             n >= b->period && build_graph(b, b->cur)) {
@@ -306,7 +318,7 @@ lb_status lb_batch_step(lb_batch* b, long n)
             n -= b->period;
             b->cur ^= b->period_flips;
         } else {
-            bool pair = !captures && pair_at(b->t, n, b->trace_every, b->traced_pairs);
+            bool pair = b->pairs && !captures && pair_at(b->t, n, b->trace_every, b->traced_pairs);
             if (singles == 1 || (singles == 2 && pair)) {
                 --singles;
                 pair = false;

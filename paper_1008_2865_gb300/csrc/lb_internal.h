@@ -143,12 +143,6 @@ struct Fp32Launch {
 int fp32_grid_blocks(int nx, int ny, Fp32Launch L);
 cudaError_t fp32_step(const StepArgs<float>& a, Fp32Launch L, bool reduce, cudaStream_t s);
 cudaError_t fp16_step(const StepArgs<__half>& a, Fp32Launch L, bool reduce, cudaStream_t s);
-// Whether the steps of a lattice of n sites march in alternating directions
-// (down in even row chunks, up in odd ones): only when its state does not fit in
-// L2 (measured: 2% slower at 1024^2, faster from 2048^2 on). A batch replica
-// follows the same rule as the lattice run alone.
-inline bool marches_alternate(long long n) { return n * 80 > (128LL << 20); }
-
 // Batches (lb_fp32.cu kernels, lb_batch.cu host code): one launch advances many
 // replicas. tiles[k] = (replica, strip, chunk, alternate), grouped by replica in
 // each replica's own CTA order; reps[r] locates replica r's tiles and its trace ring.
@@ -181,11 +175,48 @@ struct BatchLaunch {
 };
 cudaError_t fp32_batch_step(const BatchLaunch<float>& b, bool reduce, cudaStream_t s);
 cudaError_t fp16_batch_step(const BatchLaunch<__half>& b, bool reduce, cudaStream_t s);
-// Two plain steps in one pass (lb_pair.cu), for lattices of 2^18 sites on that are not
-// held on the SMs (lb_resident.cu): below, its few long chunks take as long as two
-// launches of k_step (us per step, single and paired: 250x187 10.1 and 10.2, 512^2 10.3
-// and 9.3, 700^2 12.3 and 10.2).
-inline bool pairs_pay(long long n) { return n >= (1LL << 18); }
+// Whether the state of a lattice of n sites exceeds L2.
+inline bool beyond_l2(long long n) { return n * 80 > (128LL << 20); }
+// Whether the steps of a lattice of n sites march in alternating directions
+// (down in even row chunks, up in odd ones): only when its state does not fit in
+// L2 (measured: 2% slower at 1024^2, faster from 2048^2 on). A batch replica
+// follows the same rule as the lattice run alone.
+inline bool marches_alternate(long long n) { return beyond_l2(n); }
+
+// Two plain steps in one pass (lb_pair.cu): CTAs of kPairTH threads, two columns each, and
+// kPairCols output columns.
+constexpr int kPairTH = 64;
+constexpr int kPairCols = 2 * kPairTH - 8;
+// Columns computed in a row of nx, halo and idle lanes included: by a pair, and by a step of its
+// own in CTAs of block_x threads (block_x - 2 output columns).
+inline long long pair_columns(int nx) { return 2LL * kPairTH * ((nx + kPairCols - 1) / kPairCols); }
+inline long long single_columns(int nx, int block_x)
+{
+    return (long long)block_x * ((nx + block_x - 3) / (block_x - 2));
+}
+// Pairs are for lattices of 2^18 sites on that are not held on the SMs (lb_resident.cu):
+// below, their few long chunks take as long as two launches of k_step (us per step, single and
+// paired: 250x187 10.1 and 10.2, 512^2 10.3 and 9.3, 700^2 12.3 and 10.2). And not where a
+// last strip of few columns makes a pair compute half as many columns again as single steps do,
+// with 64 threads per CTA up to 1.7 million sites, 128 beyond. Time of paired over single
+// steps (FP32 omega 1, omega 0.8, FP16) at 2^20 sites: ratio 2 (121 columns) 1.15, 1.23, 1.20,
+// (122) 0.99, 1.07, 1.10, (5) 1.30, 1.36, 1.30; 1.5 (241) 0.94, 0.99, 1.00, and 1.05, 1.08, 1.07
+// at 2^18 sites; 1.33 (140) 0.78, 0.84, 0.84; at 2^24 sites 2 (121) 1.09, 1.19, 1.25; 1.5 (241)
+// 0.84, 0.94, 0.95.
+inline bool pairs_pay(int nx, int ny, int block_x)
+{
+    const long long n = (long long)nx * ny, pair = pair_columns(nx), single = single_columns(nx, block_x);
+    return n >= (1LL << 18) && (beyond_l2(n) ? 2 * pair <= 3 * single : 5 * pair <= 7 * single);
+}
+// A pair whose first state has a trace row adds two kernels for the row, where a reduction step
+// forms it on the way. That pays where memory traffic bounds the steps (40 steps with every
+// second state traced, paired over single, FP32 and FP16: 740^2 1.15 and 1.10, 900^2 0.96 and
+// 0.96, 1024^2 1.00 and 1.03, 1150^2 0.95 and 1.06, 1300^2 0.81 and 0.90, 2048^2 0.80 and
+// 0.80), again not with nearly half as many columns again (2^24 sites: ratio 1.5 1.02, 1.33 0.93).
+inline bool traced_pairs_pay(int nx, int ny, int block_x)
+{
+    return beyond_l2((long long)nx * ny) && 5 * pair_columns(nx) <= 7 * single_columns(nx, block_x);
+}
 // (traced: the density deviations of state t are left in a.dev)
 cudaError_t fp32_step_pair(const StepArgs<float>& a, bool traced, cudaStream_t s);
 cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t s);
@@ -193,6 +224,23 @@ cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t 
 // caller chose otherwise, so even small batches gain: 27 replicas of up to 69^2, 30.7 ->
 // 9.5 us per step; nine 512^2 57.4 -> 28.7; the 96-replica sweep 338 -> 205): `tiles` (pair_tiles: replica, first column, first row, end row)
 // on the device; odd: some replica has an odd nx
+// Whether a batch takes pairs: from 2^16 sites on not where they compute half as many columns
+// again as single steps, over all replicas (tiles of 64 columns, paired over single: four
+// replicas of 5x20000, ratio 2, 1.05; 300 of 12x40, ratio 2, 1.05 and FP16 1.08; 500 of 5^2, 12,500
+// sites, 0.90 and 0.98).
+inline bool batch_pairs_pay(long long sites, long long pair, long long single)
+{
+    return sites < (1LL << 16) || 5 * pair <= 7 * single;
+}
+// And whether these take a state with a trace row along (otherwise a reduction step
+// does): not where the single steps' tiles are a few rows high anyway. Paired over single,
+// every second, fourth and tenth state traced: 5^2 FP32 1.06, 1.08, 1.02, FP16 1.12, 1.15, 1.13;
+// 16^2 0.77, 0.70, 0.65; tiles of 8 rows: 16^2 FP16 1.02, 1.04, 1.04, 64^2 FP32 0.86, 0.81, 0.77,
+// thirty 128^2 FP16 1.07, 1.02, 1.00, three 512^2 FP16 1.01, 0.97, 0.92.
+inline bool batch_traced_pairs_pay(int tallest, int tile_rows, int elem_bytes)
+{
+    return tile_rows >= 16 ? tallest >= 16 : elem_bytes == 4 && tallest >= 32;
+}
 void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, bool om1, int num_sms,
                 std::vector<int4>& tiles);
 cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int ntiles, bool odd,
@@ -244,6 +292,18 @@ inline bool launch_refused(cudaError_t e)
 // Whether the stream takes a held launch of this lattice: one step into the idle buffers. (A
 // test for a launch without steps in the kernel costs 1% of every step at 70x45.)
 cudaError_t fp32_resident_probe(const StepArgs<float>& a, ResidentBuf& b, cudaStream_t s);
+// The fewest steps worth a held launch, by the sites of a tile: it loads them, and sorts its
+// work lists, before the first step. Calls of 2, 3, 4, 5 and 6 steps, held over single launches,
+// omega = 1: 440^2 (1344 sites) 0.91, 0.74, ..; 512^2 (1728) 1.10, 0.87, ..; 560^2 (2100)
+// 1.19, 0.96, 0.83, ..; 600^2 (2432) 1.38, 1.07, 0.91, ..; 680^2 (3096) 1.38, 1.07, 0.92, ..;
+// 720^2 (3420) 1.50, 1.17, 1.01, 0.91. Otherwise: 440^2 1.00, 0.81, ..; 512^2 1.20, 0.94, ..;
+// 560^2 1.33, 1.07, 0.95, ..; 600^2 1.49, 1.20, 1.09, 1.00, 0.94.
+inline int held_least(int tile_sites, bool om1)
+{
+    if (tile_sites <= 1400) return 2;
+    if (om1) return tile_sites <= 2150 ? 3 : tile_sites <= 3200 ? 4 : 5;
+    return tile_sites <= 1900 ? 3 : tile_sites <= 2200 ? 4 : 6;
+}
 bool resident_plan(int nx, int ny, bool om1, int num_sms, ResidentBuf& b);
 cudaError_t fp32_resident(const StepArgs<float>& a, ResidentBuf& b, int block_x, int steps,
                           cudaStream_t s);

@@ -527,7 +527,7 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
 // against 522-549 with 12 warps), otherwise 12.
 template <typename T, bool OM1>
 constexpr int kPairThreads = sizeof(T) == 2 ? 512 : 384;
-constexpr int kTH = 64;   // threads per CTA
+constexpr int kTH = kPairTH;
 
 template <typename T, int TH, bool OM1, bool ODD, bool TRACE>
 __global__ void __launch_bounds__(TH, kPairThreads<T, OM1> / TH)
