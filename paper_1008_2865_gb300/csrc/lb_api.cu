@@ -17,32 +17,31 @@ namespace lbsc {
 // Test hook: allocations left before one is made to fail (-1: never).
 static std::atomic<int> g_fail_allocs_after{-1};
 
-bool state_alloc(lb_state* s, std::vector<Buffer> buffers, bool spare_last)
+bool state_alloc(lb_state* s, std::vector<Buffer> buffers, size_t spare)
 {
-    size_t total = 0, last = 0;
-    auto leave_out_last = [&]() {
-        *buffers.back().ptr = nullptr;
-        buffers.pop_back();
-        spare_last = false;
+    const size_t needed = buffers.size() - spare;
+    auto room = [](const Buffer& b) { return guarded_size(b.bytes) + 2 * kGuardBytes; };
+    auto leave_out_spare = [&]() {
+        for (; buffers.size() > needed; buffers.pop_back()) *buffers.back().ptr = nullptr;
     };
     for (size_t k = 0; k < buffers.size(); ++k) {
         int left = g_fail_allocs_after.load();
         while (left >= 0 && !g_fail_allocs_after.compare_exchange_weak(left, left - 1)) {
         }
-        if (left == 0) {   // the hook's failure (counter is now -1: disarmed)
-            if (!spare_last || k + 1 < buffers.size()) return false;
-            leave_out_last();
-            break;
-        }
-        last = guarded_size(buffers[k].bytes) + 2 * kGuardBytes;
-        total += last;
+        if (left != 0) continue;
+        // the hook's failure (counter is now -1: disarmed)
+        if (k < needed) return false;
+        leave_out_spare();
     }
+    size_t total = 0;
+    for (const Buffer& b : buffers) total += room(b);
     void* block = nullptr;
     while (cudaMalloc(&block, total) != cudaSuccess) {
         cudaGetLastError();
-        if (!spare_last) return false;
-        leave_out_last();
-        total -= last;
+        if (buffers.size() == needed) return false;
+        leave_out_spare();
+        total = 0;
+        for (const Buffer& b : buffers) total += room(b);
     }
     // the guards: one fill over small buffers and all, otherwise one at each end and where
     // two buffers meet
@@ -461,31 +460,32 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
     s->max_cta_rows = (p->ny + kMinRows - 1) / kMinRows;
     s->partials_cap += (size_t)s->max_cta_rows;
     // the control words first, at the distances that kControlPitch states; cleared below
-    bool ok = state_alloc(s, {{(void**)&s->res, 4 * sizeof(double)},
-                              {(void**)&s->err, sizeof(int)},
-                              {(void**)&s->trace_count, sizeof(int)},
-                              {(void**)&s->flag, sizeof(int)},
-                              {(void**)&s->counter, 2 * sizeof(unsigned int)},
-                              {(void**)&s->partials, 4 * sizeof(double) * s->partials_cap},
-                              {(void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols}});
-    if (ok && p->prec == LB_FP64) {
-        ok = state_alloc(s, {{(void**)&s->f64[0], 9 * sizeof(double) * N},
-                             {(void**)&s->f64[1], 9 * sizeof(double) * N},
-                             {(void**)&s->psi64, sizeof(double) * N},
-                             {(void**)&s->rho64, sizeof(double) * N}});
-    } else if (ok) {
+    std::vector<Buffer> buffers = {{(void**)&s->res, 4 * sizeof(double)},
+                                   {(void**)&s->err, sizeof(int)},
+                                   {(void**)&s->trace_count, sizeof(int)},
+                                   {(void**)&s->flag, sizeof(int)},
+                                   {(void**)&s->counter, 2 * sizeof(unsigned int)},
+                                   {(void**)&s->partials, 4 * sizeof(double) * s->partials_cap},
+                                   {(void**)&s->trace, sizeof(double) * kTraceCap * kTraceCols}};
+    auto add = [&](auto** ptr, size_t bytes) { buffers.push_back({(void**)ptr, bytes}); };
+    if (p->prec == LB_FP64) {
+        add(&s->f64[0], 9 * sizeof(double) * N);
+        add(&s->f64[1], 9 * sizeof(double) * N);
+        add(&s->psi64, sizeof(double) * N);
+        add(&s->rho64, sizeof(double) * N);
+    } else {
         const size_t gb = elem_size(p->prec) * (size_t)g_elems(p->nx, p->ny);
-        const bool traced = p->trace_every > 0;
-        std::vector<Buffer> fields = {{&s->g[0], gb},
-                                      {&s->g[1], gb},
-                                      {(void**)&s->dpsi[0], sizeof(float) * N},
-                                      {(void**)&s->dpsi[1], sizeof(float) * N}};
-        if (traced) fields.push_back({(void**)&s->dev, sizeof(float) * N});
-        ok = state_alloc(s, fields, traced);
+        add(&s->g[0], gb);
+        add(&s->g[1], gb);
+        add(&s->dpsi[0], sizeof(float) * N);
+        add(&s->dpsi[1], sizeof(float) * N);
     }
+    // what only faster ways to step need: without the memory for it the state does without
+    const size_t needed = buffers.size();
+    if (p->prec != LB_FP64 && p->trace_every > 0) add(&s->dev, sizeof(float) * N);
     ResidentBuf& rb = s->res_buf;
     size_t words4 = 0, words2 = 0;   // bytes of the halo words
-    if (ok && alone && p->prec != LB_FP64) {
+    if (alone && p->prec != LB_FP64) {
         int sms = 0;
         const bool om1 = (float)p->omega == 1.0f;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
@@ -496,7 +496,8 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
             rb.trace_every = p->trace_every;
             words4 = sizeof(uint4) * 2 * (om1 ? 1 : 3) * (size_t)N;
             words2 = sizeof(uint2) * 2 * (size_t)N;
-            std::vector<Buffer> held = {{(void**)&rb.llm, words4}, {(void**)&rb.llp, words2}};
+            add(&rb.llm, words4);
+            add(&rb.llp, words2);
             if (p->trace_every > 0) {
                 const long long rows = (8LL << 20) / (8 * N);
                 const int least = held_least(rb.tw * rb.th, om1) + 1;   // a launch at every state traced
@@ -505,13 +506,14 @@ lb_status lbsc::state_init(lb_state** out, const lb_params* p, const double* rho
                 const size_t row_cap =
                     (size_t)fp32_grid_blocks(p->nx, p->ny, Fp32Launch{64, kMinRows, 0}) +
                     (size_t)s->max_cta_rows;
-                held.push_back({(void**)&rb.counters, sizeof(unsigned int) * (1 + (size_t)rb.max_rows)});
-                held.push_back({(void**)&rb.partials, (size_t)rb.max_rows * 4 * sizeof(double) * row_cap});
-                held.push_back({(void**)&rb.dump, (size_t)rb.max_rows * 2 * sizeof(float) * N});
+                add(&rb.counters, sizeof(unsigned int) * (1 + (size_t)rb.max_rows));
+                add(&rb.partials, (size_t)rb.max_rows * 4 * sizeof(double) * row_cap);
+                add(&rb.dump, (size_t)rb.max_rows * 2 * sizeof(float) * N);
             }
-            if (!state_alloc(s, held)) rb = ResidentBuf{};
         }
     }
+    const bool ok = state_alloc(s, buffers, buffers.size() - needed);
+    if (!rb.llm) rb = ResidentBuf{};
     if (!ok) {
         free_state(s);
         return LB_ERR_OOM;

@@ -425,14 +425,15 @@ lb_status state_init(lb_state** out, const lb_params* p, const double* rho_init,
                      bool alone);
 // Allocate buffers for a state together, each with guards on both sides (pattern written on
 // the state's stream); the usable pointers are stored in order. False, with nothing allocated,
-// if there is not the memory. spare_last: the last one is left out (nullptr) if there is
-// only memory for the others. (lb_init of a traced lattice, with an allocation for each field
-// and with one for all: 2050x1999 427 and 293 us, 512^2 341 and 242 us.)
+// if there is not the memory. The last `spare` are left out (nullptr) if there is only memory
+// for the others. (lb_init, with an
+// allocation for each of the larger buffers and with one for all: 70x45 200 and 158 us, 512^2
+// 338 and 162 us, 2050x1999 425 and 250 us.)
 struct Buffer {
     void** ptr;
     size_t bytes;
 };
-bool state_alloc(lb_state* s, std::vector<Buffer> buffers, bool spare_last = false);
+bool state_alloc(lb_state* s, std::vector<Buffer> buffers, size_t spare = 0);
 // one buffer; nullptr if there is not the memory
 inline void* state_alloc(lb_state* s, size_t bytes)
 {
