@@ -128,7 +128,8 @@ __device__ __noinline__ double exp_cr(double x)
 
 // The same result, usually after some 50 instead of 2000 FP64 operations: x = (256 m + j)
 // ln2/256 + r with |r| <= ln2/512, e^x = 2^m 2^(j/256) e^r, the table and r in two
-// doubles each and e^r - 1 by its series, whose terms from r^3 on are below 2^-31 and
+// doubles each (table-driven exp: Tang, "Table-driven implementation of the exponential function
+// in IEEE floating-point arithmetic", 1989) and e^r - 1 by its series, whose terms from r^3 on are below 2^-31 and
 // need one double only. The relative error of v + lo is below 2^-81 for |x| < 32 (sum of
 // the terms' bounds: 2^-83 for ln2/256, 2^-82 for the series' double part, 2^-83 for the
 // sums; 2^-81.96 the largest of 30,000 samples against 400-bit arithmetic). If adding
@@ -498,13 +499,6 @@ __global__ void k64_fields(const double* __restrict__ f, int nx, int ny, double*
     }
 }
 
-__global__ void k64_exp(const double* __restrict__ x, double* __restrict__ y, long long n)
-{
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n;
-         s += (long long)gridDim.x * blockDim.x)
-        y[s] = exp_cr(x[s]);
-}
-
 int grid_for(long long n, int threads = 256)
 {
     long long b = (n + threads - 1) / threads;
@@ -554,12 +548,6 @@ cudaError_t fp64_fields(const double* f, int nx, int ny, double* rho, double* ux
                         cudaStream_t s)
 {
     k64_fields<<<grid_for((long long)nx * ny), 256, 0, s>>>(f, nx, ny, rho, ux, uy);
-    return cudaGetLastError();
-}
-
-cudaError_t fp64_exp_cr(const double* x, double* y, long long n, cudaStream_t s)
-{
-    k64_exp<<<grid_for(n), 256, 0, s>>>(x, y, n);
     return cudaGetLastError();
 }
 

@@ -351,7 +351,6 @@ cudaError_t fp64_energy(const Fp64Args& a, double* partials, unsigned int* count
                         cudaStream_t s);
 cudaError_t fp64_fields(const double* f, int nx, int ny, double* rho, double* ux, double* uy,
                         cudaStream_t s);
-cudaError_t fp64_exp_cr(const double* x, double* y, long long n, cudaStream_t s);
 
 }  // namespace lbsc
 
@@ -426,9 +425,8 @@ lb_status state_init(lb_state** out, const lb_params* p, const double* rho_init,
 // Allocate buffers for a state together, each with guards on both sides (pattern written on
 // the state's stream); the usable pointers are stored in order. False, with nothing allocated,
 // if there is not the memory. The last `spare` are left out (nullptr) if there is only memory
-// for the others. (lb_init, with an
-// allocation for each of the larger buffers and with one for all: 70x45 200 and 158 us, 512^2
-// 338 and 162 us, 2050x1999 425 and 250 us.)
+// for the others. (lb_init, with an allocation for each of the larger buffers and with one for
+// all: 70x45 200 and 158 us, 512^2 338 and 162 us, 2050x1999 425 and 250 us.)
 struct Buffer {
     void** ptr;
     size_t bytes;
