@@ -93,7 +93,8 @@ __device__ __forceinline__ void force_sums2(const float2 A[5], const float2 B[5]
 // step from the hardware approximation with the residual of a fused multiply-add
 // (Markstein, "Computation of elementary functions on the IBM RISC System/6000
 // processor", 1990). Equal to __frcp_rn for every FP32 value of magnitude 2^-125 to
-// 2^125; outside (a density that has blown up) __frcp_rn itself.
+// 2^125 (tests/c/rcp_check.cu compares all of them: the approximation's error decides that, not
+// the theorem alone); outside (a density that has blown up) __frcp_rn itself.
 __device__ __forceinline__ float2 neg_rcp2(float2 x)
 {
     const float lo = fminf(fabsf(x.x), fabsf(x.y)), hi = fmaxf(fabsf(x.x), fabsf(x.y));
