@@ -57,6 +57,13 @@ def step_launches(steps):
     return n
 
 
+def launch_record(launch):
+    """How the steps are launched: lb_set_launch's (block_x, rows_per_cta) is the shape of the
+    steps that are a launch of their own and of the sums behind a trace row."""
+    return {"steps_per_launch": 1 if launch[2] else 2, "single_steps": list(launch[:2]),
+            "pipeline": ["register-prefetch", "bulk-copy rings"][launch[2]]}
+
+
 METRIC = "MLUPS and % HBM roofline (FP32 fused step, 1 GB300); adjoint+batched vs plain"
 WORKLOAD = ("{n}x{n} periodic D2Q9 two-belt Shan-Chen, FP32 (deviation storage), omega=1, "
             "G1=-5.0, G2=0.6, rho=0.7(1+-1%) seeded uniform noise (seed 7), energy+mass "
@@ -203,7 +210,8 @@ def run_batched(steps, warmup, stream, dev):
             "mlups": sites * steps / (ms_batch / 1e3) / 1e6,
             "one_by_one_mlups": sites * steps / (ms_seq / 1e3) / 1e6,
             "speedup_vs_one_by_one": ms_seq / ms_batch,
-            "launch": {"block_x": launch[0], "rows_per_cta": launch[1], "cuda_graph": bool(launch[2])},
+            "launch": {"steps_per_launch": 2, "single_steps": list(launch[:2]),
+                       "cuda_graph": bool(launch[2])},
             "launches_per_step": "1 per two steps (+2 per trace row)"}
 
 
@@ -246,7 +254,7 @@ def run_adjoint(stream, dev, T=2000, n=512):
             "adjoint_over_forward": res["adjoint_ms"] / res["forward_ms"],
             "J": J, "dJ_dG1": gG[0], "dJ_dG2": gG[1],
             "includes": "forward with checkpoints, per-segment recomputation, reverse sweep "
-                        "(2 kernels per step), gradient w.r.t. rho_init, G1, G2"}
+                        "(one launch per segment), gradient w.r.t. rho_init, G1, G2"}
 
 
 def run_fp16(steps, warmup, stream, dev, peak):
@@ -281,8 +289,7 @@ def run_fp16(steps, warmup, stream, dev, peak):
     return {"workload": WORKLOAD.format(n=NX).replace("FP32 (deviation storage)",
                                                       "FP16 deviation storage, FP32 arithmetic"),
             "mlups": NX * NY / (ms / 1e3) / 1e6, "ms_per_step": ms, "steps": steps,
-            "launch": {"block_x": launch[0], "rows_per_cta": launch[1],
-                       "pipeline": ["register-prefetch", "bulk-copy rings"][launch[2]]},
+            "launch": launch_record(launch),
             "roofline": {"bound": "issue", "bytes_per_site": per_site, "achieved": gbs, "peak": peak,
                          "unit": "GB/s", "frac": gbs / peak,
                          "roof_mlups": peak * 1e9 / per_site / 1e6}}
@@ -472,8 +479,7 @@ def run_ours(args):
             "data": "synthetic (seeded SplitMix64 noise)",
             "config": {"workload": WORKLOAD.format(n=NX), "nx": NX, "ny": NY,
                        "l2": "state 5.4 GB per replica >> 129 MB L2; no flush needed",
-                       "launch": {"block_x": launch[0], "rows_per_cta": launch[1],
-                                  "pipeline": ["register-prefetch", "bulk-copy rings"][launch[2]]},
+                       "launch": launch_record(launch),
                        "parallelism": f"replicas x{ws}"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,

@@ -1,12 +1,16 @@
-"""Launch-shape autotuner for the fused step kernel.
+"""Launch-shape autotuner for the steps that are a launch of their own.
 
-The fused kernel's only free parameters are the CTA width (block_x threads =
-block_x - 2 output columns plus a one-column halo on each side) and the
-number of output rows a CTA marches over. Narrow CTAs waste a larger share of
-lanes on halo columns; short row chunks re-read more halo rows; tall chunks
-give too few CTAs for the 152 SMs. The tuner times every candidate on the
-real lattice shape with CUDA events and keeps the fastest in a JSON cache
-keyed by GPU name, lattice shape and storage precision.
+The CTA width (block_x threads = block_x - 2 output columns plus a one-column halo on
+each side) and the number of output rows a CTA marches over are the free parameters of
+k_step, which takes the steps of lb_step(1), of captured graphs and of traced states next
+to one another; the sums behind a trace row follow the same shape. Steps that share a
+launch (two at a time, or held on the SMs) have shapes of their own, which lb_set_launch
+does not touch. Narrow CTAs waste a larger share of lanes on halo columns; short row
+chunks re-read more halo rows; tall chunks give too few CTAs for the 152 SMs. The tuner
+times every candidate on the real lattice shape with CUDA events, one step a call, and
+keeps the fastest in a JSON cache keyed by GPU name, lattice shape and storage precision.
+The bulk-copy pipeline shares no launches: it is kept only where it is also faster than
+many steps a call without it.
 
   python -m paper_1008_2865_gb300.tune 8192 8192 [fp32]
 """
@@ -63,9 +67,31 @@ def candidates(nx, ny):
     return out
 
 
+def _ms_per_step(lat, stream, steps, each):
+    """Time of `steps` steps in calls of `each`."""
+    import torch
+    e0 = torch.cuda.Event(enable_timing=True)
+    e1 = torch.cuda.Event(enable_timing=True)
+    e0.record(stream)
+    for _ in range(steps // each):
+        lat.step(each)
+    e1.record(stream)
+    e1.synchronize()
+    return e0.elapsed_time(e1) / steps
+
+
+def _pick(single, many):
+    """The shape to keep: the fastest of pipeline 0 in calls of one step, unless the fastest of
+    pipeline 1 takes many steps a call faster (many(shape): ms per step)."""
+    best = [min((s for s in single if s[2] == pipe), key=single.get, default=None) for pipe in (0, 1)]
+    if best[0] is None or best[1] is None:
+        return best[0] or best[1]
+    return best[1] if many(best[1]) < many(best[0]) else best[0]
+
+
 def tune(nx, ny, prec="fp32", steps=20, device=0, save=True, G1=-5.0, G2=0.6):
-    """Time each candidate shape for `steps` steps (including the reduction steps of a
-    10-step trace period) and return ((block_x, rows), {shape: ms_per_step})."""
+    """Time each candidate shape for `steps` single steps (including the reduction steps of a
+    10-step trace period) and return ((block_x, rows, pipeline), {shape: ms_per_step})."""
     import torch
 
     from . import Lattice, inputs
@@ -80,16 +106,16 @@ def tune(nx, ny, prec="fp32", steps=20, device=0, save=True, G1=-5.0, G2=0.6):
                 lat.set_launch(bx, rows, pipe)
             except Exception:
                 continue
-            lat.step(3)
-            lat.step((-lat.t) % 10)
-            e0 = torch.cuda.Event(enable_timing=True)
-            e1 = torch.cuda.Event(enable_timing=True)
-            e0.record(stream)
-            lat.step(steps)
-            e1.record(stream)
-            e1.synchronize()
-            table[(bx, rows, pipe)] = e0.elapsed_time(e1) / steps
-    best = min(table, key=table.get)
+            for _ in range(3 + (-lat.t - 3) % 10):
+                lat.step(1)
+            table[(bx, rows, pipe)] = _ms_per_step(lat, stream, steps, 1)
+
+        def many(shape):
+            lat.set_launch(*shape)
+            lat.step(10 + -lat.t % 10)
+            return _ms_per_step(lat, stream, steps, steps)
+
+        best = _pick(table, many)
     if save:
         with _lock:
             cache = _load_cache()
@@ -118,8 +144,8 @@ def lookup_batch(shapes, prec="fp32", device=0):
 
 
 def tune_batch(rho_list, G2_list, prec="fp32", steps=20, device=0, save=True, G1=-5.0):
-    """Time each tile shape for a batch (one launch per step over all replicas, graph
-    replay) and return ((block_x, rows), {shape: ms_per_step})."""
+    """Time each tile shape of a batch's single steps (one launch per step over all replicas, one
+    step a call) and return ((block_x, rows), {shape: ms_per_step})."""
     import torch
 
     from . import Batch
@@ -136,14 +162,9 @@ def tune_batch(rho_list, G2_list, prec="fp32", steps=20, device=0, save=True, G1
                     b.set_launch(bx, rows, 1)
                 except Exception:
                     continue
-                b.step(10)
-                e0 = torch.cuda.Event(enable_timing=True)
-                e1 = torch.cuda.Event(enable_timing=True)
-                e0.record(stream)
-                b.step(steps)
-                e1.record(stream)
-                e1.synchronize()
-                table[(bx, rows)] = e0.elapsed_time(e1) / steps
+                for _ in range(10):
+                    b.step(1)
+                table[(bx, rows)] = _ms_per_step(b, stream, steps, 1)
     best = min(table, key=table.get)
     if save:
         with _lock:
