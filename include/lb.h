@@ -105,11 +105,14 @@ lb_status lb_init(lb_state** out, const lb_params* p, const double* rho_init, vo
  * towards the Eq. 4 equilibrium at the shifted velocity u + F/(omega rho),
  * then streaming. States t with t % trace_every == 0 append a trace row.
  * Steps may share a launch: an FP32 or FP16 lattice that fits the SMs' shared memory
- * (about 690 x 690 with omega = 1) takes all n in one cooperative launch, others two
- * at a time, as does a small one whose stream has fewer SMs than that launch needs; the
- * results are those of single steps, bit for bit. In a stream capture
- * every step is a launch of its own; a graph of an even number of steps continues the
- * run whenever an even number of steps has been taken outside it since its capture.
+ * (about 690 x 690 with omega = 1) takes all n in one cooperative launch, or as many as
+ * the trace rows they append can be kept; others, and a small one whose stream has fewer
+ * SMs than that launch needs, take them two at a time where that is faster. The results
+ * are those of single steps, bit for bit. A cooperative launch starts when there is room
+ * for all of it, so small lattices on streams of their own queue for the SMs: advance many
+ * of them as a batch (lb_batch_init). In a stream capture every step is a launch of its
+ * own; a graph of an even number of steps continues the run whenever an even number of
+ * steps has been taken outside it since its capture.
  * Asynchronous. Errors: LB_ERR_ARG (n < 0), LB_ERR_STATE, LB_ERR_CUDA. */
 lb_status lb_step(lb_state* s, long n);
 
@@ -241,9 +244,10 @@ lb_status lb_objective(lb_state* s, const double* rho_target, double* J);
  * rho_ref and initial density; all with the same prec — LB_FP32 or
  * LB_FP16_DELTA —, trace_every and device), e.g. a G2 sweep with distinct
  * seeds. lb_batch_step advances all of them: one persistent launch per two steps
- * (one, where a step is left over) strides over a work list of every replica's
- * tiles, and steps are replayed from a CUDA graph of one trace period when the
- * batch time is aligned to it.
+ * (one, where a step is left over or pairs would be slower) strides over a work list of
+ * every replica's tiles, and steps are replayed from a CUDA graph of one trace period
+ * when the batch time is aligned to it (until steps of the batch have been captured by
+ * the caller).
  * A replica's fields, energies and trace are bit-identical to those of the
  * same lattice run alone with the same launch shape (register-prefetch
  * pipeline). The paper runs its A2 scan (Sec. 4) as separate simulations;

@@ -2,8 +2,9 @@
 // lattices (replicas of possibly different sizes and couplings, e.g. a G2
 // sweep with distinct seeds) advanced together, one launch per two steps over a
 // work list of all replicas' tiles (k_step2_batch in lb_pair.cu; k_step_batch in
-// lb_fp32.cu where a step is left over), replayed from a CUDA graph of one trace period. Each replica is an lb_state, so
-// energies, fields and traces reuse the single-lattice code.
+// lb_fp32.cu where a step is left over or pairs do not pay), replayed from a CUDA graph of
+// one trace period. Each replica is an lb_state, so energies, fields and traces reuse the
+// single-lattice code.
 #include <algorithm>
 #include <new>
 #include <vector>
@@ -132,7 +133,7 @@ lb_status build_tables(lb_batch* b)
     b->pairs = batch_pairs_pay(sites, pair, single);
     b->traced_pairs = kept && batch_traced_pairs_pay(tallest, b->rows, (int)elem_size(b->prec));
     std::vector<int4> pair_list;
-    pair_tiles(sizes, (int)elem_size(b->prec), b->om1, b->num_sms, pair_list);
+    pair_tiles(sizes, (int)elem_size(b->prec), b->num_sms, pair_list);
     b->npair_tiles = (int)pair_list.size();
     for (BatchRep& ri : info) ri.first_row += b->ntiles;
     const bool ok =

@@ -129,10 +129,11 @@ __device__ __noinline__ double exp_cr(double x)
 // The same result, usually after some 50 instead of 2000 FP64 operations: x = (256 m + j)
 // ln2/256 + r with |r| <= ln2/512, e^x = 2^m 2^(j/256) e^r, the table and r in two
 // doubles each (table-driven exp: Tang, "Table-driven implementation of the exponential function
-// in IEEE floating-point arithmetic", 1989) and e^r - 1 by its series, whose terms from r^3 on are below 2^-31 and
-// need one double only. The relative error of v + lo is below 2^-81 for |x| < 32 (sum of
-// the terms' bounds: 2^-83 for ln2/256, 2^-82 for the series' double part, 2^-83 for the
-// sums; 2^-81.96 the largest of 30,000 samples against 400-bit arithmetic). If adding
+// in IEEE floating-point arithmetic", 1989) and e^r - 1 by its series, whose terms from r^3 on
+// are below 2^-31 and need one double only. The relative error of v + lo is below 2^-81 for
+// |x| < 32 (sum of the terms' bounds: 2^-83 for ln2/256, 2^-82 for the series' double part,
+// 2^-83 for the sums; 2^-81.96 the largest of 30,000 samples against 400-bit arithmetic;
+// tests/test_gpu_exp.py compares the rounded results). If adding
 // 2^-78 either way rounds alike, that is the correctly rounded value; otherwise (about
 // once in 2^24) exp_cr decides. (Rounding test: Ziv, "Fast evaluation of elementary
 // mathematical functions with correctly rounded last bit", 1991.)

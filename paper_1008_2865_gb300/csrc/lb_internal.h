@@ -222,8 +222,9 @@ cudaError_t fp32_step_pair(const StepArgs<float>& a, bool traced, cudaStream_t s
 cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t s);
 // The same for a batch of any size (its single-step tiles are 32 rows high unless the
 // caller chose otherwise, so even small batches gain: 27 replicas of up to 69^2, 30.7 ->
-// 9.5 us per step; nine 512^2 57.4 -> 28.7; the 96-replica sweep 338 -> 205): `tiles` (pair_tiles: replica, first column, first row, end row)
-// on the device; odd: some replica has an odd nx
+// 9.5 us per step; nine 512^2 57.4 -> 28.6; the 96-replica sweep 338 -> 178): `tiles`
+// (pair_tiles: replica, first column, first row, end row) on the device; odd: some replica
+// has an odd nx
 // Whether a batch takes pairs: from 2^16 sites on not where they compute half as many columns
 // again as single steps, over all replicas (tiles of 64 columns, paired over single: four
 // replicas of 5x20000, ratio 2, 1.05; 300 of 12x40, ratio 2, 1.05 and FP16 1.08; 500 of 5^2, 12,500
@@ -241,7 +242,7 @@ inline bool batch_traced_pairs_pay(int tallest, int tile_rows, int elem_bytes)
 {
     return tile_rows >= 16 ? tallest >= 16 : elem_bytes == 4 && tallest >= 32;
 }
-void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, bool om1, int num_sms,
+void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, int num_sms,
                 std::vector<int4>& tiles);
 cudaError_t fp32_batch_pair(const BatchLaunch<float>& b, const int4* tiles, int ntiles, bool odd,
                             bool traced, cudaStream_t s);

@@ -525,12 +525,12 @@ __device__ __forceinline__ void pair_tile(const StepArgs<T>& a, const PackedArgs
 // Resident threads per SM the registers are cut for: 16 warps where the kernel fits
 // 128 registers (FP16; with omega != 1 8 bytes are spilled, 494 us per step at 8192^2
 // against 522-549 with 12 warps), otherwise 12.
-template <typename T, bool OM1>
+template <typename T>
 constexpr int kPairThreads = sizeof(T) == 2 ? 512 : 384;
 constexpr int kTH = kPairTH;
 
 template <typename T, int TH, bool OM1, bool ODD, bool TRACE>
-__global__ void __launch_bounds__(TH, kPairThreads<T, OM1> / TH)
+__global__ void __launch_bounds__(TH, kPairThreads<T> / TH)
     k_step2(const StepArgs<T> a, const PackedArgs k, int rows)
 {
     __shared__ PairShared<T, TH, OM1> sh;
@@ -545,10 +545,10 @@ __global__ void __launch_bounds__(TH, kPairThreads<T, OM1> / TH)
 // 316 rows, 532 with one of 631; 6000^2, 334 rows: 263 with one, 268 with two). At
 // least 8 rows.
 template <typename T>
-int pair_rows(int nx, int ny, bool om1)
+int pair_rows(int nx, int ny)
 {
-    const int strips = (nx + 2 * kTH - 9) / (2 * kTH - 8);
-    const int slots = 152 * ((om1 ? kPairThreads<T, true> : kPairThreads<T, false>) / kTH);
+    const int strips = (nx + kPairCols - 1) / kPairCols;
+    const int slots = 152 * (kPairThreads<T> / kTH);
     auto rows_for = [&](int waves) {
         const int chunks = slots * waves / strips;
         return chunks > 1 ? (ny + chunks - 1) / chunks : ny;
@@ -575,9 +575,9 @@ cudaError_t with_flags(bool om1, bool odd, bool traced, F f)
 template <typename T>
 cudaError_t launch_pair(const StepArgs<T>& a, bool traced, cudaStream_t s)
 {
-    constexpr int W = 2 * kTH - 8;
+    constexpr int W = kPairCols;
     const bool om1 = a.omega == 1.0f;
-    const int rows = pair_rows<T>(a.nx, a.ny, om1);
+    const int rows = pair_rows<T>(a.nx, a.ny);
     const dim3 grid((a.nx + W - 1) / W, (a.ny + rows - 1) / rows);
     return with_flags(om1, a.nx & 1, traced, [&](auto o, auto d, auto t) {
         k_step2<T, kTH, decltype(o)::value, decltype(d)::value, decltype(t)::value>
@@ -590,7 +590,7 @@ cudaError_t launch_pair(const StepArgs<T>& a, bool traced, cudaStream_t s)
 // first column, first row, end row) of every replica. The replica's arguments are
 // staged in shared memory by warp 0 when the replica changes.
 template <typename T, bool OM1, bool ODD, bool TRACE>
-__global__ void __launch_bounds__(kTH, kPairThreads<T, OM1> / kTH)
+__global__ void __launch_bounds__(kTH, kPairThreads<T> / kTH)
     k_step2_batch(const StepArgs<T>* __restrict__ args, const int4* __restrict__ tiles, int ntiles)
 {
     __shared__ PairShared<T, kTH, OM1> sh;
@@ -622,7 +622,7 @@ template <typename T>
 cudaError_t launch_batch_pair(const BatchLaunch<T>& b, const int4* tiles, int ntiles, bool odd,
                               bool traced, cudaStream_t s)
 {
-    const int per_sm = (b.om1 ? kPairThreads<T, true> : kPairThreads<T, false>) / kTH;
+    const int per_sm = kPairThreads<T> / kTH;
     const int grid = ntiles < per_sm * b.num_sms ? ntiles : per_sm * b.num_sms;
     return with_flags(b.om1, odd, traced, [&](auto o, auto d, auto t) {
         k_step2_batch<T, decltype(o)::value, decltype(d)::value, decltype(t)::value>
@@ -637,12 +637,11 @@ cudaError_t launch_batch_pair(const BatchLaunch<T>& b, const int4* tiles, int nt
 // the height is the one that makes the estimated time least: waves of resident CTAs,
 // each as long as its tallest tile plus nine rows (the two half-busy ends of a tile
 // and its prologue).
-void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, bool om1, int num_sms,
+void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, int num_sms,
                 std::vector<int4>& tiles)
 {
-    constexpr int W = 2 * kTH - 8;
-    const int threads = elem_bytes == 2 ? (om1 ? kPairThreads<__half, true> : kPairThreads<__half, false>)
-                                        : (om1 ? kPairThreads<float, true> : kPairThreads<float, false>);
+    constexpr int W = kPairCols;
+    const int threads = elem_bytes == 2 ? kPairThreads<__half> : kPairThreads<float>;
     const long long slots = (long long)(threads / kTH) * num_sms;
     auto chunks_of = [](int ny, int rows) { return (ny + rows - 1) / rows; };
     int tallest = 8;
