@@ -17,10 +17,49 @@ namespace lbsc {
 // Test hook: allocations left before one is made to fail (-1: never).
 static std::atomic<int> g_fail_allocs_after{-1};
 
+// Allocate blocks of at most kBlockBytes for whole buffers in order (a larger buffer is a
+// block of its own) and set up their guards; nothing is allocated if that fails.
+static bool alloc_blocks(lb_state* s, const std::vector<Buffer>& buffers)
+{
+    const size_t had_allocs = s->allocs.size(), had_blocks = s->blocks.size();
+    auto room = [](const Buffer& b) { return guarded_size(b.bytes) + 2 * kGuardBytes; };
+    bool ok = true;
+    for (size_t k = 0; ok && k < buffers.size();) {
+        size_t end = k + 1, total = room(buffers[k]);
+        while (end < buffers.size() && total + room(buffers[end]) <= kBlockBytes)
+            total += room(buffers[end++]);
+        void* block = nullptr;
+        ok = cudaMalloc(&block, total) == cudaSuccess;
+        if (!ok) break;
+        s->blocks.push_back(block);
+        // the guards: one fill over small buffers and all, otherwise one at each end and
+        // where two buffers meet
+        char* at = static_cast<char*>(block);
+        auto fill = [&](char* p, size_t n) {
+            ok = ok && cudaMemsetAsync(p, kGuardByte, n, s->stream) == cudaSuccess;
+        };
+        const bool small = total <= (64u << 10);
+        fill(at, small ? total : kGuardBytes);
+        for (; k < end; ++k) {
+            const size_t body = guarded_size(buffers[k].bytes);
+            *buffers[k].ptr = at + kGuardBytes;
+            s->allocs.push_back({at, body});
+            if (!small) fill(at + kGuardBytes + body, (k + 1 < end ? 2 : 1) * kGuardBytes);
+            at += body + 2 * kGuardBytes;
+        }
+    }
+    if (ok) return true;
+    cudaGetLastError();
+    for (size_t k = had_blocks; k < s->blocks.size(); ++k) cudaFree(s->blocks[k]);
+    s->blocks.resize(had_blocks);
+    s->allocs.resize(had_allocs);
+    for (const Buffer& b : buffers) *b.ptr = nullptr;
+    return false;
+}
+
 bool state_alloc(lb_state* s, std::vector<Buffer> buffers, size_t spare)
 {
     const size_t needed = buffers.size() - spare;
-    auto room = [](const Buffer& b) { return guarded_size(b.bytes) + 2 * kGuardBytes; };
     auto leave_out_spare = [&]() {
         for (; buffers.size() > needed; buffers.pop_back()) *buffers.back().ptr = nullptr;
     };
@@ -33,42 +72,10 @@ bool state_alloc(lb_state* s, std::vector<Buffer> buffers, size_t spare)
         if (k < needed) return false;
         leave_out_spare();
     }
-    size_t total = 0;
-    for (const Buffer& b : buffers) total += room(b);
-    void* block = nullptr;
-    while (cudaMalloc(&block, total) != cudaSuccess) {
-        cudaGetLastError();
-        if (buffers.size() == needed) return false;
-        leave_out_spare();
-        total = 0;
-        for (const Buffer& b : buffers) total += room(b);
-    }
-    // the guards: one fill over small buffers and all, otherwise one at each end and where
-    // two buffers meet
-    char* at = static_cast<char*>(block);
-    bool ok = true;
-    auto fill = [&](char* p, size_t n) {
-        ok = ok && cudaMemsetAsync(p, kGuardByte, n, s->stream) == cudaSuccess;
-    };
-    const bool small = total <= (64u << 10);
-    fill(at, small ? total : kGuardBytes);
-    const size_t had = s->allocs.size();
-    for (size_t k = 0; k < buffers.size(); ++k) {
-        const size_t body = guarded_size(buffers[k].bytes);
-        *buffers[k].ptr = at + kGuardBytes;
-        s->allocs.push_back({at, body});
-        if (!small) fill(at + kGuardBytes + body, (k + 1 < buffers.size() ? 2 : 1) * kGuardBytes);
-        at += body + 2 * kGuardBytes;
-    }
-    if (!ok) {
-        cudaGetLastError();
-        cudaFree(block);
-        s->allocs.resize(had);
-        for (const Buffer& b : buffers) *b.ptr = nullptr;
-        return false;
-    }
-    s->blocks.push_back(block);
-    return true;
+    if (alloc_blocks(s, buffers)) return true;
+    if (buffers.size() == needed) return false;
+    leave_out_spare();
+    return alloc_blocks(s, buffers);
 }
 
 Couplings couplings(double G1, double G2)

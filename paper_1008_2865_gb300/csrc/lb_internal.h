@@ -426,8 +426,10 @@ lb_status state_init(lb_state** out, const lb_params* p, const double* rho_init,
 // Allocate buffers for a state together, each with guards on both sides (pattern written on
 // the state's stream); the usable pointers are stored in order. False, with nothing allocated,
 // if there is not the memory. The last `spare` are left out (nullptr) if there is only memory
-// for the others. (lb_init, with an allocation for each of the larger buffers and with one for
-// all: 70x45 200 and 158 us, 512^2 338 and 162 us, 2050x1999 425 and 250 us.)
+// for the others. They share blocks of up to kBlockBytes (lb_init, with an allocation for each
+// of the larger buffers and with one for all: 70x45 200 and 158 us, 512^2 338 and 162 us, 2050x1999
+// 425 and 250 us, but 8192^2 1390 and 2100 us).
+constexpr size_t kBlockBytes = size_t(1) << 30;
 struct Buffer {
     void** ptr;
     size_t bytes;
