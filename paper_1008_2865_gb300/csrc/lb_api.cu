@@ -335,9 +335,10 @@ lb_status step_streamed(lb_state* s, long n, bool pairs)
 {
     const int te = s->p.trace_every;
     const bool bulk = s->launch.pipeline == 1;
-    pairs = pairs && pairs_pay(s->p.nx, s->p.ny, s->launch.block_x);
+    pairs = pairs && pairs_pay(s->p.nx, s->p.ny, s->launch.block_x, (int)elem_size(s->p.prec));
     // one pair fewer if the buffers would not swap as single steps swap them
-    const bool traced = s->dev && traced_pairs_pay(s->p.nx, s->p.ny, s->launch.block_x);
+    const bool traced = s->dev && traced_pairs_pay(s->p.nx, s->p.ny, s->launch.block_x,
+                                                   (int)elem_size(s->p.prec));
     int singles = pairs && s->in_graphs && pairs_made(s->t, n, te, traced) % 2 != 0 ? 2 : 0;
     while (n > 0) {
         const bool reduce = te > 0 && s->t % te == 0;

@@ -120,21 +120,25 @@ lb_status build_tables(lb_batch* b)
     b->nrows = nrows_total;
     std::vector<std::pair<int, int>> sizes;
     int tallest = 0;
-    long long sites = 0, pair = 0, single = 0;
+    double sites = 0.0, pair = 0.0, single = 0.0;
     bool kept = true;                   // every replica can keep a traced state's deviations
     for (const lb_state* s : b->reps) {
         sizes.emplace_back(s->p.nx, s->p.ny);
         tallest = std::max(tallest, s->p.ny);
         kept = kept && s->dev;
-        sites += s->N;
-        pair += pair_columns(s->p.nx) * s->p.ny;
-        single += single_columns(s->p.nx, b->block_x) * s->p.ny;
+        sites += (double)s->N;
+        pair += (double)pair_columns(s->p.nx) * s->p.ny;
+        single += (double)single_columns(s->p.nx, b->block_x) * s->p.ny;
     }
-    b->pairs = batch_pairs_pay(sites, pair, single);
-    b->traced_pairs = kept && batch_traced_pairs_pay(tallest, b->rows, (int)elem_size(b->prec));
     std::vector<int4> pair_list;
     pair_tiles(sizes, (int)elem_size(b->prec), b->num_sms, pair_list);
     b->npair_tiles = (int)pair_list.size();
+    BatchWork w{b->ntiles, b->block_x, std::min(b->rows, tallest), b->npair_tiles, 0,
+                (int)elem_size(b->prec), b->num_sms};
+    for (const int4& t : pair_list) w.pair_chunk = std::max(w.pair_chunk, t.w - t.z);
+    const double estimate = batch_paired_over_single(w);
+    b->pairs = batch_pairs_pay(b->block_x, b->rows, sites / single, estimate);
+    b->traced_pairs = kept && batch_traced_pairs_pay(b->block_x, b->rows, tallest, pair / single, estimate);
     for (BatchRep& ri : info) ri.first_row += b->ntiles;
     const bool ok =
         (b->prec == LB_FP32 ? upload_args<float>(b) : upload_args<__half>(b)) &&

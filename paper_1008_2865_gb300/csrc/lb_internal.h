@@ -197,25 +197,33 @@ inline long long single_columns(int nx, int block_x)
 // Pairs are for lattices of 2^18 sites on that are not held on the SMs (lb_resident.cu):
 // below, their few long chunks take as long as two launches of k_step (us per step, single and
 // paired: 250x187 10.1 and 10.2, 512^2 10.3 and 9.3, 700^2 12.3 and 10.2). And not where a
-// last strip of few columns makes a pair compute half as many columns again as single steps do,
+// last strip of few columns makes a pair compute that many more columns than single steps do,
 // with 64 threads per CTA up to 1.7 million sites, 128 beyond. Time of paired over single
-// steps (FP32 omega 1, omega 0.8, FP16) at 2^20 sites: ratio 2 (121 columns) 1.15, 1.23, 1.20,
-// (122) 0.99, 1.07, 1.10, (5) 1.30, 1.36, 1.30; 1.5 (241) 0.94, 0.99, 1.00, and 1.05, 1.08, 1.07
-// at 2^18 sites; 1.33 (140) 0.78, 0.84, 0.84; at 2^24 sites 2 (121) 1.09, 1.19, 1.25; 1.5 (241)
-// 0.84, 0.94, 0.95.
-inline bool pairs_pay(int nx, int ny, int block_x)
+// steps (FP32 with omega 1 and 0.8, FP16 alike) by that ratio:
+//   450,000 sites: 1.33 (140 columns) held, 1.08, held, 0.93; 1.0 (360) held, 0.84, ..
+//   600,000: 1.5 (241) 1.00, 1.07, 1.14, 1.12; 1.33 (140) 0.82, 0.88, 0.94, 0.95; 1.0 0.80 to 1.00
+//   10^6: 2 (121) 1.15, 1.23, 1.20; 1.5 (241) 0.91, 0.96, 1.11, 1.00; 1.33 0.82, 0.87, 0.87, 0.84
+//   1.3 million: 1.5 (241) 0.88, 0.96, 1.04, 0.99, (246) 0.80, 0.88, 0.95, 0.92
+//   2^24: 2 (121) 1.09, 1.19, 1.25; 1.5 (241) 0.84, 0.94, 0.95; 1.0 0.57 to 0.69
+inline bool pairs_pay(int nx, int ny, int block_x, int elem_bytes)
 {
     const long long n = (long long)nx * ny, pair = pair_columns(nx), single = single_columns(nx, block_x);
-    return n >= (1LL << 18) && (beyond_l2(n) ? 2 * pair <= 3 * single : 5 * pair <= 7 * single);
+    return n < (1LL << 18)                            ? false
+           : n < (1LL << 19)                          ? 4 * pair <= 5 * single
+           : n < (elem_bytes == 4 ? 900000 : 1200000) ? 5 * pair <= 7 * single
+                                                      : 2 * pair <= 3 * single;
 }
 // A pair whose first state has a trace row adds two kernels for the row, where a reduction step
-// forms it on the way. That pays where memory traffic bounds the steps (40 steps with every
-// second state traced, paired over single, FP32 and FP16: 740^2 1.15 and 1.10, 900^2 0.96 and
-// 0.96, 1024^2 1.00 and 1.03, 1150^2 0.95 and 1.06, 1300^2 0.81 and 0.90, 2048^2 0.80 and
-// 0.80), again not with nearly half as many columns again (2^24 sites: ratio 1.5 1.02, 1.33 0.93).
-inline bool traced_pairs_pay(int nx, int ny, int block_x)
+// forms it on the way. That pays where memory traffic bounds the steps (every second state
+// traced, paired over single, FP32 and FP16: 740^2 1.15 and 1.10, 900^2 0.96 and 0.96, 1024^2 1.00
+// and 1.03, 1024x1269 0.95 and 1.07, 1024x1562 0.84 and 0.97, 1300^2 0.81 and 0.90, 2048^2 0.80 and
+// 0.80), again not with that many more columns (ratio 1.14, 425 columns, 1.3 million sites 1.03 and
+// 1.14, 1.6 million 0.94 and 1.05; 2^24 sites: ratio 1.5 1.02, 1.33 0.93).
+inline bool traced_pairs_pay(int nx, int ny, int block_x, int elem_bytes)
 {
-    return beyond_l2((long long)nx * ny) && 5 * pair_columns(nx) <= 7 * single_columns(nx, block_x);
+    const long long n = (long long)nx * ny, pair = pair_columns(nx), single = single_columns(nx, block_x);
+    return beyond_l2(n) ? 5 * pair <= 7 * single
+                        : n >= (elem_bytes == 4 ? 1250000 : 1500000) && 5 * pair <= 6 * single;
 }
 // (traced: the density deviations of state t are left in a.dev)
 cudaError_t fp32_step_pair(const StepArgs<float>& a, bool traced, cudaStream_t s);
@@ -225,22 +233,46 @@ cudaError_t fp16_step_pair(const StepArgs<__half>& a, bool traced, cudaStream_t 
 // 9.5 us per step; nine 512^2 57.4 -> 28.6; the 96-replica sweep 338 -> 178): `tiles`
 // (pair_tiles: replica, first column, first row, end row) on the device; odd: some replica
 // has an odd nx
-// Whether a batch takes pairs: from 2^16 sites on not where they compute half as many columns
-// again as single steps, over all replicas (tiles of 64 columns, paired over single: four
-// replicas of 5x20000, ratio 2, 1.05; 300 of 12x40, ratio 2, 1.05 and FP16 1.08; 500 of 5^2, 12,500
-// sites, 0.90 and 0.98).
-inline bool batch_pairs_pay(long long sites, long long pair, long long single)
+// Estimated time of a batch's pair over that of two single steps. Either takes its CTAs' rows
+// one after another, a row in the longer of its latency and the SM's share of the work:
+// fitted to 1,200 batches of 2 to 500 lattices from 5^2 to 122x2000 at six shapes (FP32 and
+// FP16 separately for the pair), within 10% and 6% on average.
+struct BatchWork {
+    int tiles, block_x, chunk;        // of the single step; chunk: rows of its tallest CTA
+    int pair_tiles, pair_chunk;       // of the pair
+    int elem_bytes, num_sms;
+};
+inline double batch_paired_over_single(const BatchWork& w)
 {
-    return sites < (1LL << 16) || 5 * pair <= 7 * single;
+    auto most = [](double x, double y) { return x > y ? x : y; };
+    const bool half = w.elem_bytes == 2;
+    const double warps = w.tiles * (w.block_x / 32.0) / w.num_sms;
+    const double single = 4.0 + (w.chunk + 2) * most(0.8, 0.06 * warps);
+    const int slots = (half ? 8 : 6) * w.num_sms, waves = (w.pair_tiles + slots - 1) / slots;
+    const double pair_warps = 2.0 * w.pair_tiles / w.num_sms;
+    const double pair = half ? 6.0 + (w.pair_chunk + 5) * most(1.1 * waves, 0.15 * pair_warps)
+                             : 6.0 + (w.pair_chunk + 7) * most(0.7 * waves, 0.14 * pair_warps);
+    return pair / (2.0 * single);
 }
-// And whether these take a state with a trace row along (otherwise a reduction step
-// does): not where the single steps' tiles are a few rows high anyway. Paired over single,
-// every second, fourth and tenth state traced: 5^2 FP32 1.06, 1.08, 1.02, FP16 1.12, 1.15, 1.13;
-// 16^2 0.77, 0.70, 0.65; tiles of 8 rows: 16^2 FP16 1.02, 1.04, 1.04, 64^2 FP32 0.86, 0.81, 0.77,
-// thirty 128^2 FP16 1.07, 1.02, 1.00, three 512^2 FP16 1.01, 0.97, 0.92.
-inline bool batch_traced_pairs_pay(int tallest, int tile_rows, int elem_bytes)
+// Whether a batch takes pairs. With the default tiles of single steps (126 columns, 32 rows) and
+// larger ones always: paired over single 0.96 at most (two 5^2, FP16), 0.27 at best; nor do
+// 62 columns of 32 rows change that (0.94 at most) unless nearly all of them are idle (fill: sites
+// over the columns that single steps compute; 5x20000 up to 1.21). Otherwise the estimate
+// decides: where it allows pairs they take 1.00 at most, where it does not up to 1.44 (500 of
+// 12x40 in tiles of 62x8) and 0.79 at best.
+inline bool batch_pairs_pay(int block_x, int rows, double fill, double estimate)
 {
-    return tile_rows >= 16 ? tallest >= 16 : elem_bytes == 4 && tallest >= 32;
+    return (rows >= 32 && (block_x >= 128 || fill >= 0.15)) || estimate <= 1.0;
+}
+// And whether these take a state with a trace row along (otherwise a reduction step does). Not
+// lattices of a few rows (every second state traced: 5^2 1.02 to 1.17, 16^2 0.75), and with
+// smaller tiles only by a margin, or where a pair computes few columns more: allowed 1.06 at
+// most, otherwise up to 1.45. column_ratio: of pair_columns to single_columns, over all rows.
+inline bool batch_traced_pairs_pay(int block_x, int rows, int tallest, double column_ratio,
+                                   double estimate)
+{
+    return tallest >= 16 && ((block_x >= 128 && rows >= 32) || column_ratio <= 1.25 ||
+                             estimate <= (rows >= 32 ? 0.9 : 0.7));
 }
 void pair_tiles(const std::vector<std::pair<int, int>>& sizes, int elem_bytes, int num_sms,
                 std::vector<int4>& tiles);

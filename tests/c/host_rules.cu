@@ -38,34 +38,54 @@ static void wait_limit()
 static void shared_launches()
 {
     // pairs: enough sites, and not for a second strip of two columns
-    expect(pairs_pay(760, 760, 64) && pairs_pay(2050, 1999, 128) && pairs_pay(140, 7490, 64) &&
-               pairs_pay(64, 16384, 64) && pairs_pay(241, 17404, 128) && pairs_pay(5, 3355444, 128),
+    expect(pairs_pay(760, 760, 64, 4) && pairs_pay(2050, 1999, 128, 4) && pairs_pay(140, 7490, 64, 4) &&
+               pairs_pay(64, 16384, 64, 4) && pairs_pay(246, 5284, 64, 2) && pairs_pay(241, 4149, 64, 4) && pairs_pay(241, 17404, 128, 4) &&
+               pairs_pay(5, 3355444, 128, 4),
            "pairs");
-    expect(!pairs_pay(500, 500, 64) && !pairs_pay(122, 8000, 64) && !pairs_pay(121, 138655, 128) &&
-               !pairs_pay(5, 52429, 64) && !pairs_pay(8, 40000, 64) && !pairs_pay(241, 1200, 64),
+    expect(!pairs_pay(500, 500, 64, 4) && !pairs_pay(122, 8000, 64, 4) && !pairs_pay(121, 138655, 128, 4) &&
+               !pairs_pay(5, 52429, 64, 4) && !pairs_pay(8, 40000, 64, 4) && !pairs_pay(241, 2489, 64, 4) && !pairs_pay(241, 4149, 64, 2) &&
+               !pairs_pay(140, 3214, 64, 4),
            "no pairs");
-    // traced states in pairs: beyond L2
-    expect(traced_pairs_pay(1300, 1300, 128) && traced_pairs_pay(8192, 8192, 128) &&
-               traced_pairs_pay(361, 46475, 128),
+    // traced states in pairs: beyond L2 or nearly
+    expect(traced_pairs_pay(1300, 1300, 128, 2) && traced_pairs_pay(8192, 8192, 128, 4) &&
+               traced_pairs_pay(361, 46475, 128, 4) && traced_pairs_pay(1024, 1269, 64, 4) &&
+               traced_pairs_pay(1024, 1562, 64, 2),
            "traced pairs");
-    expect(!traced_pairs_pay(740, 740, 64) && !traced_pairs_pay(1150, 1150, 64) &&
-               !traced_pairs_pay(122, 34380, 128) && !traced_pairs_pay(241, 69616, 128),
+    expect(!traced_pairs_pay(740, 740, 64, 4) && !traced_pairs_pay(1024, 1269, 64, 2) &&
+               !traced_pairs_pay(1024, 1024, 64, 4) && !traced_pairs_pay(122, 34380, 128, 4) &&
+               !traced_pairs_pay(241, 69616, 128, 4),
            "no traced pairs");
-    auto batch = [](int count, int nx, int ny, int block_x) {
-        return batch_pairs_pay((long long)count * nx * ny, pair_columns(nx) * ny * count,
-                               single_columns(nx, block_x) * ny * count);
+    // batches: {pairs, traced pairs} of `count` lattices at a shape of their single steps
+    auto batch = [](int count, int nx, int ny, int block_x, int rows, int elem_bytes) {
+        std::vector<std::pair<int, int>> sizes(count, {nx, ny});
+        std::vector<int4> tiles;
+        pair_tiles(sizes, elem_bytes, 152, tiles);
+        const int strips = (nx + block_x - 3) / (block_x - 2);
+        BatchWork w{count * strips * ((ny + rows - 1) / rows), block_x, rows < ny ? rows : ny,
+                    (int)tiles.size(), 0, elem_bytes, 152};
+        for (const int4& t : tiles) w.pair_chunk = t.w - t.z > w.pair_chunk ? t.w - t.z : w.pair_chunk;
+        const double e = batch_paired_over_single(w);
+        return std::make_pair(batch_pairs_pay(block_x, rows, (double)nx / single_columns(nx, block_x), e),
+                              batch_traced_pairs_pay(block_x, rows, ny,
+                                                     (double)pair_columns(nx) / single_columns(nx, block_x), e));
     };
-    expect(batch(96, 64, 64, 128) && batch(500, 5, 5, 64) && batch(4, 5, 20000, 128) &&
-               batch(12, 130, 640, 64),
-           "pairs of a batch");
-    expect(!batch(4, 5, 20000, 64) && !batch(300, 12, 40, 64) && !batch(8, 122, 2000, 64),
-           "no pairs of a batch");
-    expect(batch_traced_pairs_pay(640, 32, 4) && batch_traced_pairs_pay(16, 32, 2) &&
-               batch_traced_pairs_pay(64, 8, 4),
-           "traced pairs of a batch");
-    expect(!batch_traced_pairs_pay(5, 32, 4) && !batch_traced_pairs_pay(16, 8, 4) &&
-               !batch_traced_pairs_pay(128, 8, 2),
-           "no traced pairs of a batch");
+    const struct {
+        int count, nx, ny, block_x, rows, elem_bytes;
+        bool pairs, traced;
+    } batches[] = {{74, 125, 75, 128, 32, 2, true, true},   {8, 122, 2000, 128, 32, 4, true, true},
+                   {9, 512, 512, 128, 32, 4, true, true},   {96, 64, 64, 64, 8, 4, true, true},
+                   {200, 5, 5, 128, 32, 4, true, false},    {500, 5, 5, 64, 8, 2, true, false},
+                   {24, 16, 16, 64, 32, 2, true, true},     {30, 128, 128, 64, 8, 2, true, false},
+                   {2, 5, 20000, 128, 32, 4, true, true},   {8, 5, 20000, 64, 32, 4, false, false},
+                   {500, 12, 40, 64, 8, 4, false, false},   {500, 37, 37, 64, 16, 4, false, false},
+                   {24, 5, 400, 64, 8, 2, false, false},    {74, 125, 75, 128, 8, 2, false, false},
+                   {8, 122, 2000, 64, 32, 4, true, false},  {74, 122, 122, 64, 32, 4, true, true}};
+    for (const auto& t : batches) {
+        const auto got = batch(t.count, t.nx, t.ny, t.block_x, t.rows, t.elem_bytes);
+        std::printf("%d of %dx%d at %dx%d: ", t.count, t.nx, t.ny, t.block_x, t.rows);
+        expect(got.first == t.pairs && (got.first && got.second) == t.traced, "pairs of a batch");
+        std::printf("\n");
+    }
     // held launches of few steps: not of large tiles (152 SMs)
     const struct {
         int n;

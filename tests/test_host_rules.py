@@ -8,8 +8,8 @@ import pytest
 from paper_1008_2865_gb300 import build as lbbuild
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-# the library's units that hold a rule (resident_plan), and what they call
-UNITS = [os.path.join(lbbuild.BUILDDIR, u) for u in ("lb_resident.o", "lb_trace.o")]
+# the library's units that hold a rule (resident_plan, pair_tiles), and what they call
+UNITS = [os.path.join(lbbuild.BUILDDIR, u) for u in ("lb_resident.o", "lb_pair.o", "lb_trace.o")]
 
 
 @pytest.fixture(scope="module")
