@@ -403,7 +403,6 @@ struct Control {
     int err, trace_count, flag;
 };
 constexpr size_t kControlPitch = 3 * kGuardBytes;   // from one word to the next: guards and words
-constexpr size_t kControlBytes = 3 * kControlPitch + sizeof(int);   // res to flag
 }  // namespace lbsc
 
 // The state behind the opaque lb_state* of the C ABI (lb_api.cu owns its
